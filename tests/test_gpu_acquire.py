@@ -84,3 +84,22 @@ def test_acquire_flags_bad_ids(tiny):
     cnt = cnt.cpu().numpy()
     assert cnt[0] >= 1 and cnt[1] == -1 and cnt[2] == -1
     assert np.all(out.cpu().numpy().view(np.uint32)[1:] == NONE)
+
+
+@pytest.mark.parametrize("d,M", [(60, 33), (128, 64), (132, 64), (260, 64), (512, 64), (516, 64), (1024, 64)])
+def test_acquire_row_widths_and_chunk_edges(d, M):
+    # every row-chunk count per lane; candidate counts around the test's chunks (8 and 16) and the sort's powers of
+    # two; wide rows with M = 64 keep more rows than fit in shared memory
+    rng = np.random.default_rng(d)
+    X = rng.standard_normal((700, d)).astype(np.float32)
+    X /= np.linalg.norm(X, axis=1, keepdims=True)
+    _case(X, 60, [0, 1, 2, 7, 8, 9, 15, 16, 17, 31, 33, 64, 65, 513], M, d % 8 == 4, seed=d)
+
+
+def test_acquire_close_rows_tie():
+    # many equal distances (rows repeated): the order by id decides, and no kept row repeats
+    rng = np.random.default_rng(3)
+    X = rng.standard_normal((40, 64)).astype(np.float32)
+    X = np.repeat(X, 8, axis=0)
+    X /= np.linalg.norm(X, axis=1, keepdims=True)
+    _case(X, 40, [5, 48, 130], 32, True, seed=3)

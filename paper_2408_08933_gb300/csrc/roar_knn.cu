@@ -20,7 +20,7 @@
 #include <atomic>
 #include <cstdio>
 
-#include "roar_internal.cuh"
+#include "roar_knn_tc.cuh"
 
 namespace roar {
 
@@ -48,8 +48,7 @@ __global__ void quantize_bf16_kernel(const float *__restrict__ X, int64_t n, int
 }
 
 // One warp per row: BF16 rows padded with zeros to dp columns (the kNN
-// kernel's operands: rows of whole 64-column K chunks, so each chunk of a row
-// is one aligned 128-byte segment).
+// kernel's operands: rows of whole 16-column MMA steps).
 __global__ void quantize_bf16_pad_kernel(const float *__restrict__ X, int64_t n, int d, int dp,
                                          __nv_bfloat16 *__restrict__ out) {
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -185,10 +184,6 @@ extern "C" roar_status roar_quantize(const float *X, int64_t n, int32_t d, roar_
 }
 
 namespace roar {
-cudaError_t knn_tc_launch(const __nv_bfloat16 *T16, int64_t nt, const __nv_bfloat16 *X16, int64_t n, int d,
-                          int C, int cap, float *buf_s, uint32_t *buf_i, uint32_t *cand, int *err,
-                          uint64_t wait_ns, cudaStream_t s);
-int64_t knn_tc_wave_rows(int d);
 // Wall-time limit of each bounded wait in the tensor-core kernel: 2 s by
 // default, far above any legitimate wait there.
 constexpr int64_t kKnnWaitDefaultNs = 2000000000ll;
@@ -202,7 +197,7 @@ extern "C" roar_status roar_knn_set_wait_limit_ns(int64_t ns) {
 
 extern "C" roar_status roar_knn(const float *T, int64_t nt, const float *X, int64_t n, int32_t d,
                                 int32_t kk, uint32_t *ids, float *dist, void *stream) {
-    constexpr int C = 128, CAP = 1024;
+    constexpr int C = 128;
     if (nt < 0 || n < 1 || n >= 0x7FFFFFFF || d < 8 || d % 8 != 0 || d > 512 || kk < 1 || kk > C ||
         kk > n) {
         set_error("roar_knn: need n >= kk, 1 <= kk <= 128, d % 8 == 0, 8 <= d <= 512");
@@ -211,22 +206,26 @@ extern "C" roar_status roar_knn(const float *T, int64_t nt, const float *X, int6
     if (nt == 0) return ROAR_OK;
     if (!T || !X || !ids || !dist || !aligned(T, 16) || !aligned(X, 16)) return ROAR_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    const int dp = (d + 63) / 64 * 64;   // BF16 operand rows padded to whole 64-column K chunks
-    // Query rows per launch: whole waves of the kernel, about 131,072 at most
-    // (a partial last wave leaves SMs idle for a whole sweep of X).
-    const int64_t wave = knn_tc_wave_rows(dp);
+    const int dp = (d + 15) / 16 * 16;   // BF16 operand rows padded to whole MMA steps of K
+    // Query rows per launch: whole waves of the kernel, about 131,072 at most.
+    const int64_t wave = knn_tc_wave_rows(d);
     const int64_t RB = std::min<int64_t>(nt, std::max<int64_t>(wave, 131072 / wave * wave));
+    KnnPlan whole, rest;   // of a launch of RB rows and of the last one
     __nv_bfloat16 *t16 = nullptr, *x16 = nullptr;
-    float *bs = nullptr;
-    uint32_t *bi = nullptr, *cand = nullptr;
+    void *scratch = nullptr, *lists = nullptr;
+    uint32_t *cand = nullptr;
     int *err = nullptr;
     const uint64_t wait_ns = (uint64_t)g_knn_wait_ns.load();
     roar_status rc = ROAR_OK;
     int herr = 0;
-    cudaError_t e = cudaMalloc(&t16, (size_t)nt * dp * 2);
+    cudaError_t e = knn_tc_plan(RB, n, d, &whole);
+    if (e == cudaSuccess) e = knn_tc_plan(nt % RB ? nt % RB : RB, n, d, &rest);
+    if (e != cudaSuccess) return cuda_fail(e, "roar_knn: launch plan");
+    const size_t lists_bytes = std::max(whole.lists_bytes, rest.lists_bytes);
+    e = cudaMalloc(&t16, (size_t)nt * dp * 2);
     if (e == cudaSuccess) e = cudaMalloc(&x16, (size_t)n * dp * 2);
-    if (e == cudaSuccess) e = cudaMalloc(&bs, (size_t)RB * CAP * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&bi, (size_t)RB * CAP * 4);
+    if (e == cudaSuccess) e = cudaMalloc(&scratch, std::max(whole.scratch_bytes, rest.scratch_bytes));
+    if (e == cudaSuccess && lists_bytes) e = cudaMalloc(&lists, lists_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&cand, (size_t)RB * C * 4);
     if (e == cudaSuccess) e = cudaMalloc(&err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);
@@ -240,7 +239,7 @@ extern "C" roar_status roar_knn(const float *T, int64_t nt, const float *X, int6
     if ((rc = quantize_bf16_pad(X, n, d, dp, x16, s)) != ROAR_OK) goto done;
     for (int64_t r0 = 0; r0 < nt; r0 += RB) {
         const int64_t rb = std::min(RB, nt - r0);
-        e = knn_tc_launch(t16 + r0 * dp, rb, x16, n, dp, C, CAP, bs, bi, cand, err, wait_ns, s);
+        e = knn_tc_launch(rb == RB ? whole : rest, t16 + r0 * dp, rb, x16, n, dp, scratch, lists, cand, err, wait_ns, s);
         if (e != cudaSuccess) {
             rc = cuda_fail(e, "roar_knn: tensor-core scores");
             goto done;
@@ -263,8 +262,8 @@ extern "C" roar_status roar_knn(const float *T, int64_t nt, const float *X, int6
 done:
     cudaFree(t16);
     cudaFree(x16);
-    cudaFree(bs);
-    cudaFree(bi);
+    cudaFree(scratch);
+    cudaFree(lists);
     cudaFree(cand);
     cudaFree(err);
     return rc;

@@ -36,7 +36,7 @@ __device__ __forceinline__ bool less_entry(float da, uint32_t ia, float db, uint
     return da < db || (da == db && ia < ib);
 }
 
-// One warp per row. BF16: round to nearest even, scale 1.
+// One warp per row, any alignment. BF16: round to nearest even, scale 1.
 __global__ void quantize_bf16_kernel(const float *__restrict__ X, int64_t n, int d,
                                      __nv_bfloat16 *__restrict__ out) {
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -47,19 +47,7 @@ __global__ void quantize_bf16_kernel(const float *__restrict__ X, int64_t n, int
     for (int i = lane; i < d; i += 32) o[i] = __float2bfloat16_rn(x[i]);
 }
 
-// One warp per row: BF16 rows padded with zeros to dp columns (the kNN
-// kernel's operands: rows of whole 16-column MMA steps).
-__global__ void quantize_bf16_pad_kernel(const float *__restrict__ X, int64_t n, int d, int dp,
-                                         __nv_bfloat16 *__restrict__ out) {
-    const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (row >= n) return;
-    const float *x = X + row * d;
-    __nv_bfloat16 *o = out + row * dp;
-    for (int i = lane; i < dp; i += 32) o[i] = i < d ? __float2bfloat16_rn(x[i]) : __float2bfloat16_rn(0.0f);
-}
-
-// One warp per row. FP8-E4M3: s = maxabs / 448 (IEEE division), code = E4M3(x / s)
+// One warp per row, any alignment. FP8-E4M3: s = maxabs / 448 (IEEE division), code = E4M3(x / s)
 // rounded to nearest even and saturated to +-448; an all-zero row gets s = 1.
 __global__ void quantize_fp8_kernel(const float *__restrict__ X, int64_t n, int d,
                                     uint8_t *__restrict__ out, float *__restrict__ scales) {
@@ -76,6 +64,59 @@ __global__ void quantize_fp8_kernel(const float *__restrict__ X, int64_t n, int 
     uint8_t *o = out + row * d;
     for (int i = lane; i < d; i += 32)
         o[i] = (uint8_t)__nv_cvt_float_to_fp8(__fdiv_rn(x[i], s), __NV_SATFINITE, __NV_E4M3);
+}
+
+// The same for 16-byte-aligned rows, bound by HBM: LPR lanes per row (a power of
+// two, so narrow rows fill the warp too), each element read once, 16 bytes per
+// lane and load. Measured on GB300, 1M x 512 to FP8: 486 us (5.3 TB/s) with a
+// second read of the row and one-byte stores, 363 us (7.0 TB/s) so.
+
+// BF16 rows of d4 16-byte chunks into rows of dp4 8-byte ones, zeros past d4.
+template <int LPR>
+__global__ void __launch_bounds__(256) quantize_bf16_vec_kernel(const float4 *__restrict__ X, int64_t n, int d4, int dp4,
+                                                                uint2 *__restrict__ out) {
+    const int64_t row = (int64_t)blockIdx.x * (256 / LPR) + threadIdx.x / LPR;
+    if (row >= n) return;
+    const float4 *x = X + row * d4;
+    uint2 *o = out + row * dp4;
+#pragma unroll 4
+    for (int c = threadIdx.x % LPR; c < dp4; c += LPR) {
+        const float4 v = c < d4 ? __ldcs(x + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+        o[c] = make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
+    }
+}
+
+// FP8 rows of d4 chunks, at most LPR * NCH, held in registers between the row's
+// maximum and the codes.
+template <int LPR, int NCH>
+__global__ void __launch_bounds__(256) quantize_fp8_vec_kernel(const float4 *__restrict__ X, int64_t n, int d4,
+                                                               uint32_t *__restrict__ out, float *__restrict__ scales) {
+    const int64_t row = (int64_t)blockIdx.x * (256 / LPR) + threadIdx.x / LPR;
+    const int l = threadIdx.x % LPR;
+    float4 v[NCH];
+    float m = 0.0f;
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+        const int ch = l + LPR * c;
+        v[c] = row < n && ch < d4 ? __ldcs(X + row * d4 + ch) : make_float4(0.f, 0.f, 0.f, 0.f);
+        m = fmaxf(m, fmaxf(fmaxf(fabsf(v[c].x), fabsf(v[c].y)), fmaxf(fabsf(v[c].z), fabsf(v[c].w))));
+    }
+#pragma unroll
+    for (int o = LPR / 2; o >= 1; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
+    if (row >= n) return;
+    const float s = (m == 0.0f) ? 1.0f : __fdiv_rn(m, 448.0f);
+    if (l == 0) scales[row] = s;
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+        const int ch = l + LPR * c;
+        if (ch >= d4) break;
+        const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(__fdiv_rn(v[c].x, s), __fdiv_rn(v[c].y, s)),
+                                                     __NV_SATFINITE, __NV_E4M3);
+        const uint32_t hi = __nv_cvt_float2_to_fp8x2(make_float2(__fdiv_rn(v[c].z, s), __fdiv_rn(v[c].w, s)),
+                                                     __NV_SATFINITE, __NV_E4M3);
+        out[row * d4 + ch] = lo | (hi << 16);
+    }
 }
 
 // Exact FP32 re-scoring of C candidates per query row, then the first kk in
@@ -152,10 +193,33 @@ __global__ void rescore_kernel(const float *__restrict__ T, int64_t nt, const fl
 
 }  // namespace
 
+// BF16 copy in rows of dp >= d columns (zeros past d); X 16-byte and out 8-byte aligned.
+static cudaError_t quantize_bf16_vec(const float *X, int64_t n, int d, int dp, void *out, cudaStream_t s) {
+    const int d4 = d / 4, dp4 = dp / 4;
+    const float4 *x = reinterpret_cast<const float4 *>(X);
+    uint2 *o = reinterpret_cast<uint2 *>(out);
+    if (dp4 <= 8) quantize_bf16_vec_kernel<8><<<(unsigned)((n + 31) / 32), 256, 0, s>>>(x, n, d4, dp4, o);
+    else if (dp4 <= 16) quantize_bf16_vec_kernel<16><<<(unsigned)((n + 15) / 16), 256, 0, s>>>(x, n, d4, dp4, o);
+    else quantize_bf16_vec_kernel<32><<<(unsigned)((n + 7) / 8), 256, 0, s>>>(x, n, d4, dp4, o);
+    return cudaGetLastError();
+}
+
+static cudaError_t quantize_fp8_vec(const float *X, int64_t n, int d, void *out, float *scales, cudaStream_t s) {
+    const int d4 = d / 4;
+    const float4 *x = reinterpret_cast<const float4 *>(X);
+    uint32_t *o = reinterpret_cast<uint32_t *>(out);
+    const unsigned rows8 = (unsigned)((n + 7) / 8);
+    if (d4 <= 8) quantize_fp8_vec_kernel<8, 1><<<(unsigned)((n + 31) / 32), 256, 0, s>>>(x, n, d4, o, scales);
+    else if (d4 <= 16) quantize_fp8_vec_kernel<16, 1><<<(unsigned)((n + 15) / 16), 256, 0, s>>>(x, n, d4, o, scales);
+    else if (d4 <= 32) quantize_fp8_vec_kernel<32, 1><<<rows8, 256, 0, s>>>(x, n, d4, o, scales);
+    else if (d4 <= 64) quantize_fp8_vec_kernel<32, 2><<<rows8, 256, 0, s>>>(x, n, d4, o, scales);
+    else if (d4 <= 128) quantize_fp8_vec_kernel<32, 4><<<rows8, 256, 0, s>>>(x, n, d4, o, scales);
+    else quantize_fp8_vec_kernel<32, 8><<<rows8, 256, 0, s>>>(x, n, d4, o, scales);
+    return cudaGetLastError();
+}
+
 roar_status quantize_bf16_pad(const float *X, int64_t n, int d, int dp, void *out, cudaStream_t s) {
-    const int64_t blocks = (n + 7) / 8;
-    quantize_bf16_pad_kernel<<<(unsigned)blocks, 256, 0, s>>>(X, n, d, dp, (__nv_bfloat16 *)out);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = quantize_bf16_vec(X, n, d, dp, out, s);
     return e == cudaSuccess ? ROAR_OK : cuda_fail(e, "quantize_bf16");
 }
 
@@ -171,15 +235,20 @@ extern "C" roar_status roar_quantize(const float *X, int64_t n, int32_t d, roar_
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t blocks = (n + 7) / 8;
     if (blocks > 0x7FFFFFFF) return ROAR_EINVAL;
-    if (dtype == ROAR_BF16) {
+    cudaError_t e = cudaSuccess;
+    // Rows are multiples of 16 bytes, so the first one's alignment is every one's.
+    if (dtype == ROAR_BF16 && aligned(X, 16) && aligned(out, 8)) {
+        e = quantize_bf16_vec(X, n, d, d, out, s);
+    } else if (dtype == ROAR_BF16) {
         quantize_bf16_kernel<<<(unsigned)blocks, 256, 0, s>>>(X, n, d, (__nv_bfloat16 *)out);
     } else if (dtype == ROAR_FP8_E4M3) {
         if (!scales) return ROAR_EINVAL;
-        quantize_fp8_kernel<<<(unsigned)blocks, 256, 0, s>>>(X, n, d, (uint8_t *)out, scales);
+        if (aligned(X, 16) && aligned(out, 4)) e = quantize_fp8_vec(X, n, d, out, scales, s);
+        else quantize_fp8_kernel<<<(unsigned)blocks, 256, 0, s>>>(X, n, d, (uint8_t *)out, scales);
     } else {
         return ROAR_EINVAL;
     }
-    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     return e == cudaSuccess ? ROAR_OK : cuda_fail(e, "roar_quantize");
 }
 

@@ -320,7 +320,7 @@ cudaError_t launch_acquire(const float *X, int64_t n, int d, const uint32_t *xs,
     const size_t smem = (size_t)scap * d * 4 + (size_t)keycap * 8;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kAcqRowBytes + 8 * kAcqMaxCand);   // any launch's
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, 32 * W, smem);
     if (e != cudaSuccess) return e;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(nx, (int64_t)sms * std::max(1, per)));

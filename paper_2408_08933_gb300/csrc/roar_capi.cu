@@ -261,7 +261,6 @@ roar_status plan_search(roar_index *idx, int32_t lmax, SearchArgs &a, int &block
     a.dtype = (int32_t)idx->dtype;
     a.lcap = (lmax + 31) / 32 * 32;
     a.max_visits = idx->max_visits;
-    a.hash_log2 = t.hash == 0 ? hash_log2_for(lmax) : (t.hash < 0 ? 0 : t.hash);
     a.bi_off = idx->bi_off;
     a.bi_q = idx->bi_q;
     a.bi_nt = idx->bi_nt;
@@ -271,7 +270,8 @@ roar_status plan_search(roar_index *idx, int32_t lmax, SearchArgs &a, int &block
         set_error("roar_search: the bipartite-graph search runs one warp per query");
         return ROAR_EINVAL;
     }
-    int bps = search_blocks_per_sm((int)idx->dtype, idx->d, idx->rmax, a.lcap, a.hash_log2, tw, bi);
+    choose_visited(a, t.hash, tw, lmax, nq, idx->num_sms);
+    int bps = search_blocks_per_sm(a, tw);
     if (bps <= 0) {
         set_error("roar_search: this L does not fit in shared memory");
         return ROAR_EINVAL;

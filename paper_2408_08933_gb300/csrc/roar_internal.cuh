@@ -12,7 +12,8 @@ constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr uint32_t kChecked = 0x80000000u;   // pool entry already expanded
 constexpr uint32_t kIdMask = 0x7FFFFFFFu;
 constexpr int kWarpsPerBlock = 4;            // one query per warp, 4 per CTA
-constexpr int kCandCap = ROAR_MAX_RMAX;      // new neighbours per hop, at most rmax
+// New neighbours per hop, at most rmax: candidate buffer slots.
+__host__ __device__ constexpr int cand_cap(int rmax) { return rmax <= 64 ? 64 : ROAR_MAX_RMAX; }
 constexpr int kMaxWarpsPerSm = 32;
 #ifndef ROAR_MIN_BLOCKS
 #define ROAR_MIN_BLOCKS 4
@@ -64,6 +65,10 @@ struct SearchArgs {
     int32_t lcap;            // pool capacity, multiple of 32, >= every L
     uint32_t max_visits;
     int32_t hash_log2;       // shared-memory visited-table slots, log2 (0: none)
+    int32_t ct_log2;         // compact visited table: 16-bit slots, log2 (0: none; then hash_log2 is 0)
+    int32_t ct_rem;          // ... bits of an id's permuted value kept in its slot
+    uint32_t ct_mask;        // ... 2^(bits of n - 1) - 1, the domain of the permutation
+    int32_t staged;          // row gathers staged in shared memory (one-warp kernels)
     uint32_t *vbits;         // per-warp-slot visited bitmaps, vbits_words each, all-zero at rest
     int64_t vbits_words;
     uint32_t *vlog;          // per-warp-slot log of the ids set in the bitmap, vlog_cap each
@@ -102,10 +107,11 @@ struct SearchArgs {
     int32_t trace_cap;
 };
 
-// Shared memory of one warp: pool (8 B per slot), candidate buffers (16 B per
-// slot), optional visited table (4 B per slot).
-__host__ __device__ inline size_t search_smem_per_warp(int lcap, int hash_log2) {
-    return (size_t)lcap * 8 + (size_t)kCandCap * 16 + (hash_log2 ? ((size_t)4 << hash_log2) : 0);
+// The compact visited table: 2^ct_log2 16-bit slots in buckets of 16 (32
+// bytes), and one byte per bucket counting its slots taken.
+constexpr int kCtBucketLog2 = 4;
+__host__ __device__ inline size_t ct_bytes(int ct_log2) {
+    return ct_log2 ? ((size_t)2 << ct_log2) + ((size_t)1 << (ct_log2 - kCtBucketLog2)) : 0;
 }
 
 // 16-byte row chunks a lane holds: rows of d floats are d/4 chunks dealt to
@@ -156,29 +162,32 @@ __host__ __device__ inline size_t stage_bytes(int dtype, int S, int d4) {
 // Rows are copied in 16-byte pieces, so a row's bytes must be a multiple of 16
 // (FP32: any d % 4 == 0; BF16: d % 8 == 0; FP8: d % 16 == 0).
 __host__ __device__ inline bool search_staged(int dtype, int d, int tw, int lcap) {
-    return tw == 1 && lcap <= ROAR_STAGE_MAX_LCAP && stage_rows(dtype, 1) > 0 &&
+    return tw == 1 && search_nch(d) == 2 && lcap <= ROAR_STAGE_MAX_LCAP && stage_rows(dtype, 2) > 0 &&
            ((size_t)d * (4 >> dtype)) % 16 == 0;
 }
-__host__ __device__ inline size_t search_stage_bytes(int dtype, int d, int tw, int lcap) {
-    if (!search_staged(dtype, d, tw, lcap)) return 0;
-    return stage_bytes(dtype, stage_rows(dtype, search_nch(d)), d >> 2);
-}
 
-// Per team: the above plus a 16-byte control block (claimed query, hop count,
-// pool size), then `stage` bytes of gather staging.
-__host__ __device__ inline size_t search_smem_per_team(int lcap, int hash_log2, size_t stage = 0) {
-    return search_smem_per_warp(lcap, hash_log2) + 16 + stage;
+// Shared memory of one team: pool (8 B per slot), candidate buffers (16 B per
+// slot), optional visited table (4 B per slot), a 16-byte control block
+// (claimed query, hop count, pool size), optional compact visited table, then
+// `stage` bytes of gather staging.
+__host__ __device__ inline size_t search_smem_per_team(const SearchArgs &a, size_t stage) {
+    return (size_t)a.lcap * 8 + (size_t)cand_cap(a.rmax) * 16 + (a.hash_log2 ? ((size_t)4 << a.hash_log2) : 0) + 16 +
+           ct_bytes(a.ct_log2) + stage;
 }
-// Resident CTAs per SM for this configuration with teams of tw warps (0 if it
+// Resident CTAs per SM for this launch with teams of tw warps (0 if it
 // cannot launch), the teams per CTA, and the launch itself.
-int search_blocks_per_sm(int dtype, int d, int rmax, int lcap, int hash_log2, int tw, bool bi = false);
+int search_blocks_per_sm(const SearchArgs &a, int tw);
 int teams_per_block(int tw);
 cudaError_t launch_search(const SearchArgs &a, int blocks, int tw, cudaStream_t s, bool configure = true);
 template <int DT>
 const void *kernel_table(int nch, int rpl, int tw, bool staged);
 const void *kernel_table_bi(int nch, int rpl);
 
-int hash_log2_for(int L);
+// Picks the visited set (hash_log2, ct_log2 and what belongs to it) and the
+// gather of a launch of nq queries of beam width up to L, with teams of tw
+// warps on sms SMs; hash: 0 automatic, -1 bitmap only, else a shared table of
+// 2^hash slots.
+void choose_visited(SearchArgs &a, int hash, int tw, int L, int64_t nq, int sms);
 
 // Fills a SearchArgs for a handle (index rows, tuning, scratch sized for the
 // full resident grid) and picks blocks and team warps. Defined in roar_capi.cu.

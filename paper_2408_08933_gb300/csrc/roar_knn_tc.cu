@@ -984,7 +984,8 @@ bool make_map(CUtensorMap *m, const __nv_bfloat16 *base, int64_t rows, int dp, i
 
 // CTA pairs that run at once (one CTA per SM).
 cudaError_t resident_pairs(size_t smem, int *pairs) {
-    cudaError_t e = cudaFuncSetAttribute(knn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(knn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         222 * 1024);   // the most any width needs: calls of several threads share it
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2);

@@ -110,8 +110,8 @@ extern "C" roar_status roar_search_noalloc(int64_t n, int32_t d, const float *ba
     a.dtype = ROAR_F32;
     a.lcap = (L + 31) / 32 * 32;
     a.max_visits = max_visits;
-    a.hash_log2 = hash_log2_for(L);
-    const int bps = search_blocks_per_sm(ROAR_F32, d, rmax, a.lcap, a.hash_log2, 1);
+    choose_visited(a, 0, 1, L, nq, sms);
+    const int bps = search_blocks_per_sm(a, 1);
     if (bps <= 0) {
         set_error("roar_search_noalloc: this L does not fit in shared memory");
         return ROAR_EINVAL;

@@ -1,6 +1,9 @@
 // Beam-search dispatch: kernel choice, shared-memory sizing, occupancy and launch.
 // The kernels themselves are in roar_search_kernel.cuh (one translation unit
 // per traversal type).
+#include <algorithm>
+#include <cmath>
+
 #include "roar_internal.cuh"
 
 namespace roar {
@@ -15,11 +18,11 @@ int threads_for(int tw) { return 32 * (tw > kWarpsPerBlock ? tw : kWarpsPerBlock
 
 int teams_per_block(int tw) { return threads_for(tw) / (32 * tw); }
 
-const void *search_kernel(int dtype, int d, int rmax, int tw, int lcap, bool bi = false) {
-    const int nch = nch_for(d), rpl = rmax <= 64 ? 2 : 4;
-    if (bi) return (dtype == 0 && tw == 1) ? kernel_table_bi(nch, rpl) : nullptr;
-    const bool staged = search_staged(dtype, d, tw, lcap);
-    switch (dtype) {
+static const void *search_kernel(const SearchArgs &a, int tw) {
+    const int nch = nch_for(a.d), rpl = a.rmax <= 64 ? 2 : 4;
+    if (a.bi_off) return (a.dtype == 0 && tw == 1) ? kernel_table_bi(nch, rpl) : nullptr;
+    const bool staged = a.staged != 0;
+    switch (a.dtype) {
         case 0: return kernel_table<0>(nch, rpl, tw, staged);
         case 1: return kernel_table<1>(nch, rpl, tw, staged);
         case 2: return kernel_table<2>(nch, rpl, tw, staged);
@@ -27,28 +30,22 @@ const void *search_kernel(int dtype, int d, int rmax, int tw, int lcap, bool bi 
     }
 }
 
-int hash_log2_for(int L) {
-    // Measured on GB300 (1M x 200, 10k queries, FP32 / BF16 / FP8): the
-    // global bitmap alone is faster from L = 20 on (15-20 % at L = 60-90); the
-    // shared table only helps the shortest searches.
-    if (L >= 16) return 0;
-    const int lcap = (L + 31) / 32 * 32;
-    const size_t budget = (size_t)(228 - kMinBlocksPerSm) * 1024;  // per SM, minus per-CTA reserve
-    int lg = 10;
-    while ((1 << lg) < 32 * L && lg < 14) ++lg;
-    // Keep kMinBlocksPerSm CTAs resident; below 2^9 slots use the bitmap alone.
-    while (lg >= 9 && search_smem_per_team(lcap, lg) * kWarpsPerBlock * kMinBlocksPerSm > budget) --lg;
-    return lg >= 9 ? lg : 0;
+static size_t stage_of(const SearchArgs &a) {
+    return a.staged ? stage_bytes(a.dtype, stage_rows(a.dtype, search_nch(a.d)), a.d >> 2) : 0;
 }
 
-int search_blocks_per_sm(int dtype, int d, int rmax, int lcap, int hash_log2, int tw, bool bi) {
-    const void *fn = search_kernel(dtype, d, rmax, tw, lcap, bi);
+// Shared memory a CTA can have. A kernel is allowed all of it, never the size
+// of one launch: launches of other sizes by other threads share the kernel.
+constexpr size_t kMaxSmem = 227 * 1024;
+static cudaError_t allow_smem(const void *fn) {
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+}
+
+int search_blocks_per_sm(const SearchArgs &a, int tw) {
+    const void *fn = search_kernel(a, tw);
     if (!fn) return 0;
-    const size_t stage = bi ? 0 : search_stage_bytes(dtype, d, tw, lcap);
-    const size_t smem = search_smem_per_team(lcap, hash_log2, stage) * teams_per_block(tw);
-    if (smem > 227 * 1024) return 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return 0;
+    const size_t smem = search_smem_per_team(a, stage_of(a)) * teams_per_block(tw);
+    if (smem > kMaxSmem || allow_smem(fn) != cudaSuccess) return 0;
     int blocks = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, threads_for(tw), smem) != cudaSuccess)
         return 0;
@@ -56,15 +53,62 @@ int search_blocks_per_sm(int dtype, int d, int rmax, int lcap, int hash_log2, in
     return blocks < cap ? blocks : cap;
 }
 
+// Visited rows of one query of beam width L, about (measured on 1M rows of
+// d = 200 and 512: 592 / 2,899 / 4,343 / 7,430 / 11,498 at L = 10 / 100 / 200 /
+// 500 / 1000; fewer on smaller sets).
+static double visits_for(int L) { return 128.0 * std::pow((double)L, 2.0 / 3.0); }
+
+void choose_visited(SearchArgs &a, int hash, int tw, int L, int64_t nq, int sms) {
+    a.hash_log2 = hash > 0 ? hash : 0;
+    a.ct_log2 = 0;
+    a.staged = 0;
+    if (hash == 0) {
+        // The compact table: twice the visits expected, or less, as long as the
+        // CTAs this launch can use stay resident. Measured on GB300, 1M rows,
+        // 10,000 queries, against the bitmap alone: FP32 d = 200 L = 100 4.99 ms
+        // (bitmap 6.01, a larger table with fewer CTAs 5.61), L = 500 17.0
+        // (18.6); BF16 d = 200 L = 100 4.64 (5.21); FP8 4.78 (4.99). It has to
+        // hold a quarter of the visits to help (FP8 L = 350 with 1,024 slots
+        // 12.23, bitmap 12.13), and two thirds while the bitmaps of all warps fit
+        // half of L2 (100k rows, FP32 L = 200 3.81 / 3.92, L = 500 8.94 / 8.68).
+        const int bps = search_blocks_per_sm(a, tw), tpb = teams_per_block(tw);
+        const int64_t need = (nq + (int64_t)tpb * sms - 1) / ((int64_t)tpb * sms);
+        const int64_t want = std::min<int64_t>(std::max<int64_t>(need, 1), bps);
+        const double est = std::min(visits_for(L), (double)a.n);
+        int lg = 9;
+        while (lg < 15 && (double)(1 << lg) < 2.0 * est) ++lg;
+        auto resident = [&](int x) {
+            a.ct_log2 = x;
+            const size_t smem = search_smem_per_team(a, 0) * tpb;
+            return smem > kMaxSmem ? 0 : (int64_t)(228 * 1024 / (smem + 1024));
+        };
+        while (lg >= 9 && resident(lg) < want) --lg;
+        a.ct_log2 = 0;
+        int bits = 1;   // of the ids
+        while (bits < 31 && ((int64_t)1 << bits) < a.n) ++bits;
+        const double bitmaps = (double)std::min<int64_t>(nq, want * tpb * sms) * (double)a.n / 8.0;
+        const double share = bitmaps <= 64.0 * (1 << 20) ? 1.5 : 4.0;
+        const int bucket_bits = lg - kCtBucketLog2;
+        if (lg >= 9 && (double)(1 << lg) * share >= est && bits - bucket_bits <= 16) {   // a slot keeps 16 bits
+            if (bits < bucket_bits) bits = bucket_bits;
+            a.ct_log2 = lg;
+            a.ct_rem = bits - bucket_bits;
+            a.ct_mask = (uint32_t)(((uint64_t)1 << bits) - 1);
+        }
+    }
+    // The staged gather pays only without the compact table, whose bytes it
+    // would need (with it 5.1-5.4 ms at L = 100), and for 129 to 256 columns (d =
+    // 512, L = 100: 8.5 ms staged, 7.2 not; d = 100: 2.39, 2.35).
+    if (!a.ct_log2 && !a.bi_off) a.staged = search_staged(a.dtype, a.d, tw, a.lcap) ? 1 : 0;
+}
+
 cudaError_t launch_search(const SearchArgs &a, int blocks, int tw, cudaStream_t s, bool configure) {
-    const bool bi = a.bi_off != nullptr;
-    const void *fn = search_kernel(a.dtype, a.d, a.rmax, tw, a.lcap, bi);
+    const void *fn = search_kernel(a, tw);
     if (!fn || blocks <= 0) return cudaErrorInvalidValue;
-    const size_t stage = bi ? 0 : search_stage_bytes(a.dtype, a.d, tw, a.lcap);
-    const size_t smem = search_smem_per_team(a.lcap, a.hash_log2, stage) * teams_per_block(tw);
+    const size_t smem = search_smem_per_team(a, stage_of(a)) * teams_per_block(tw);
     cudaError_t e = cudaSuccess;
     if (configure) {  // already done by search_blocks_per_sm when planning
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(fn);
         if (e != cudaSuccess) return e;
     }
     e = cudaMemsetAsync(a.work, 0, sizeof(unsigned int), s);

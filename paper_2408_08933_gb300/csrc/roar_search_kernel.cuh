@@ -4,12 +4,16 @@
 //
 // Per warp, in shared memory: the size-L candidate pool sorted by
 // (distance, id) with an "expanded" bit in each id, the new candidates of the
-// current hop, and optionally a small exact visited table (open addressing,
-// linear probing). Once that table would pass half load, or when it is
-// disabled, the visited set continues in a per-warp bitmap in global memory
-// (one bit per base row, set with one atomicOr round trip); every id set
-// there is appended to a per-warp log, and at the end of the query the log
-// clears exactly those words, so the bitmap is all-zero between queries.
+// current hop, and the visited set: usually a compact exact table of 16-bit
+// slots (CompactTable), or by tuning a small table of ids (open addressing,
+// linear probing) or none. What a table cannot take goes to a per-warp bitmap
+// in global memory (one bit per base row, set with one atomicOr round trip):
+// ids whose bucket of the compact table is full; every id once a table of ids
+// would pass half load. Ids set there are appended to a per-warp log, and at
+// the end of the query the log clears exactly those words, so the bitmap is
+// all-zero between queries. (The bitmaps of all warps are far larger than L2:
+// with them alone a hop waited for atomics on DRAM lines, and their lines were a
+// fifth of the FP32 search's DRAM traffic, more than the rows' for FP8.)
 //
 // Each hop: pick the first unexpanded pool entry, read its adjacency row
 // (coalesced, one id per lane), test-and-insert the neighbours into the
@@ -110,6 +114,15 @@ __device__ __forceinline__ void prefetch_rows_l2(const void *base, uint32_t rowb
     }
 }
 
+// The same for one row, by one lane: for BF16 / FP8 rows fewer instructions than
+// spreading the lines (d = 512, L = 350: 9.37 -> 8.75 ms); FP32 rows were 2-3 %
+// slower with it.
+__device__ __forceinline__ void prefetch_row_l2(const void *base, uint32_t rowbytes, uint32_t u) {
+    const char *p = static_cast<const char *>(base) + (size_t)u * rowbytes;
+    const char *line = reinterpret_cast<const char *>(reinterpret_cast<uintptr_t>(p) & ~(uintptr_t)127);
+    for (; line < p + rowbytes; line += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(line));
+}
+
 // Raw 4-element chunk of a row in the traversal format.
 template <int DT>
 struct RawChunk;
@@ -187,6 +200,7 @@ __host__ __device__ constexpr int rerank_rows() {
 template <int DT, int NCH>
 __host__ __device__ constexpr int batch_rows() {
     constexpr int f32 = NCH >= ROAR_BATCH_CHUNKS ? 1 : ROAR_BATCH_CHUNKS / NCH;
+    if (DT == 0 && NCH == 2) return 5;   // (L = 90: 4.39 ms; 4, 6, 7, 8 rows 4.52, 4.52, 4.58, 4.65)
     constexpr int lowp = 2 * f32 > ROAR_LOWP_MAX_ROWS ? (f32 > ROAR_LOWP_MAX_ROWS ? f32 : ROAR_LOWP_MAX_ROWS) : 2 * f32;
     return DT == 0 ? f32 : lowp;
 }
@@ -407,55 +421,66 @@ __device__ __forceinline__ int smem_visit(uint32_t *tab, int log2, uint32_t u, b
     return 3;
 }
 
-// Insert (cd_, ci_) at slot pos of a sorted pool of `size` entries with
-// capacity L (pos < L, pos <= size): slots pos.. move up by one and the last
-// falls off a full pool. Works on groups of 4 slots per lane (16-byte shared
-// accesses, 128 slots per step) from the top down; the slot that crosses
-// into the group above comes from the next lane by a shuffle (or, for the
-// lowest group of a step, from shared memory below the step, not yet moved).
-__device__ __forceinline__ void pool_insert_one(float *pd, uint32_t *pi, int size, int L, int pos,
-                                                float cd_, uint32_t ci_, int lane) {
-    const int last = min(size, L - 1);  // highest destination slot
-    const int g_lo = pos >> 2, g_hi = last >> 2;
-    float4 *pd4 = reinterpret_cast<float4 *>(pd);
-    uint4 *pi4 = reinterpret_cast<uint4 *>(pi);
-    for (int gb = g_hi; gb >= g_lo; gb -= 32) {
-        const int g = gb - lane;
-        const bool act = g >= g_lo;
-        float4 dv = make_float4(0.f, 0.f, 0.f, 0.f);
-        uint4 iv = make_uint4(0u, 0u, 0u, 0u);
-        if (act) {
-            dv = pd4[g];
-            iv = pi4[g];
-        }
-        float pdv = __shfl_down_sync(kFull, dv.w, 1);
-        uint32_t piv = __shfl_down_sync(kFull, iv.w, 1);
-        if (act && (lane == 31 || g - 1 < g_lo) && g > 0) {
-            pdv = pd[4 * g - 1];
-            piv = pi[4 * g - 1];
-        }
-        if (act) {
-            const int i0 = 4 * g;
-            float4 nd = dv;
-            uint4 ni = iv;
-            // destination slot i takes the old slot i - 1 for pos < i <= last, the new entry at pos
-#define ROAR_SLOT(J, PREVD, PREVI, DST_D, DST_I)                   \
-    {                                                               \
-        const int i = i0 + J;                                       \
-        if (i == pos) { DST_D = cd_; DST_I = ci_; }                 \
-        else if (i > pos && i <= last) { DST_D = PREVD; DST_I = PREVI; } \
+// Exact visited set of one query in 16-bit slots. An id below 2^b (b: the bits
+// of n - 1) is permuted within its b bits by an odd multiplier; the top bits of
+// the result pick a bucket of 16 slots and the rest, at most 16 bits, is what
+// a slot keeps, so (bucket, slot value) stands for exactly one id at half the
+// bytes of a table of ids. Slots of a bucket fill in order (0xFFFF: free), so a
+// bucket is full when its last slot is taken; ids that find theirs full, and
+// those whose value is 0xFFFF, go to the global bitmap. An id is therefore in
+// the bitmap only if its bucket is full or its value is 0xFFFF. Measured on
+// GB300, 1M x 200, 10,000 queries, L = 90: FP32 5.32 -> 4.39 ms.
+struct CompactTable {
+    uint4 *slots;            // two per bucket
+    uint32_t *taken;         // a byte per bucket
+    uint32_t mask;
+    int rem, log2;
+    __device__ __forceinline__ CompactTable(unsigned char *p, const SearchArgs &a)
+        : slots(reinterpret_cast<uint4 *>(p)),
+          taken(reinterpret_cast<uint32_t *>(p + (a.ct_log2 ? ((size_t)2 << a.ct_log2) : 0))),
+          mask(a.ct_mask), rem(a.ct_rem), log2(a.ct_log2) {}
+    __device__ __forceinline__ void clear(int lane) const {
+        const int n4 = 1 << (log2 - 3);            // 16-byte pieces
+        for (int i = lane; i < n4; i += 32) slots[i] = make_uint4(kNone, kNone, kNone, kNone);
+        const int nb = 1 << (log2 - kCtBucketLog2 - 2);   // words of bucket counts
+        for (int i = lane; i < nb; i += 32) taken[i] = 0u;
     }
-            ROAR_SLOT(0, pdv, piv, nd.x, ni.x)
-            ROAR_SLOT(1, dv.x, iv.x, nd.y, ni.y)
-            ROAR_SLOT(2, dv.y, iv.y, nd.z, ni.z)
-            ROAR_SLOT(3, dv.z, iv.z, nd.w, ni.w)
-#undef ROAR_SLOT
-            pd4[g] = nd;
-            pi4[g] = ni;
+    // Nonzero if one of the two halves of v is zero.
+    static __device__ __forceinline__ uint32_t zero_half(uint32_t v) { return (v - 0x00010001u) & ~v & 0x80008000u; }
+    // The whole warp: test-and-insert of u in the lanes with `want`. True where
+    // u was not yet visited and is now; to_bits where the bitmap has to decide.
+    __device__ __forceinline__ bool visit(uint32_t u, bool want, bool &to_bits) const {
+        const int lane = threadIdx.x & 31;
+        // The same id twice in a row of the graph: the lowest lane has it.
+        const unsigned same = __match_any_sync(kFull, want ? u : (0x80000000u | (uint32_t)lane));
+        bool fresh = false;
+        to_bits = false;
+        if (want && lane == __ffs(same) - 1) {
+            const uint32_t h = (u * 2654435769u) & mask;
+            const uint32_t b = h >> rem, v = h & ((1u << rem) - 1u), pat = v | (v << 16);
+            const uint4 x = slots[2 * b], y = slots[2 * b + 1];
+            const uint32_t hit = zero_half(x.x ^ pat) | zero_half(x.y ^ pat) | zero_half(x.z ^ pat) |
+                                 zero_half(x.w ^ pat) | zero_half(y.x ^ pat) | zero_half(y.y ^ pat) |
+                                 zero_half(y.z ^ pat) | zero_half(y.w ^ pat);
+            const bool special = v == 0xFFFFu;
+            if (special || !hit) {
+                to_bits = special || (y.w >> 16) != 0xFFFFu;
+                if (!to_bits) {
+                    const uint32_t sh = 8u * (b & 3u);
+                    const uint32_t slot = (atomicAdd(&taken[b >> 2], 1u << sh) >> sh) & 0xFFu;
+                    if (slot < 16u) {
+                        reinterpret_cast<uint16_t *>(slots)[16u * b + slot] = (uint16_t)v;
+                        fresh = true;
+                    } else {
+                        to_bits = true;      // other lanes of this round took the last slots
+                    }
+                }
+            }
         }
         __syncwarp();
+        return fresh;
     }
-}
+};
 
 // Global bitmap visited set: true if u was not yet set.
 __device__ __forceinline__ bool bitmap_visit(uint32_t *bits, uint32_t u) {
@@ -475,6 +500,82 @@ __device__ __forceinline__ int lower_bound_entries(const float *dv, const uint32
     return lo;
 }
 
+
+// Merges the cnt new candidates (cd, ci; ids not in the pool) into the sorted
+// pool of `size` entries and capacity L, in place; entries past L fall off.
+// Returns the new size and lowers `cursor` to the first slot that changed. 32
+// candidates at a time, one per lane: each finds its rank among them and its
+// place in the pool, hence its final slot; a bit per slot of each 32-slot row
+// then tells every slot whether it takes a candidate (the next in order) or the
+// entry as many slots back as candidates lie before it. Rows go from the top
+// down, four at a time with all reads before the writes, so nothing is
+// overwritten before it is read; a lane's accesses are to consecutive slots.
+// (Inserting up to four candidates one at a time, each moving the pool's tail,
+// and scattering the entries of larger merges after a search per entry: FP8 L =
+// 100 5.24 -> 4.95 ms, BF16 d = 512 L = 350 9.84 -> 9.37 ms, one FP32 query 543 ->
+// 454 us with this merge.)
+// (sd, si: room for 32 sorted candidates.)
+__device__ __forceinline__ int pool_merge(float *pd, uint32_t *pi, int size, int L, const float *cd,
+                                          const uint32_t *ci, int cnt, float *sd, uint32_t *si, int &cursor,
+                                          int lane) {
+    const unsigned lt = (1u << lane) - 1u;
+    for (int j0 = 0; j0 < cnt; j0 += 32) {
+        const int m = min(32, cnt - j0);
+        const bool have = lane < m;
+        const float dj = have ? cd[j0 + lane] : 0.0f;
+        const uint32_t ij = have ? ci[j0 + lane] : 0u;
+        int r = 0;
+        for (int x = 0; x < m; x += 4) {   // (buffers are multiples of 4 slots)
+            const float4 d4 = *reinterpret_cast<const float4 *>(cd + j0 + x);
+            const uint4 i4 = *reinterpret_cast<const uint4 *>(ci + j0 + x);
+            r += less_entry(d4.x, i4.x, dj, ij) ? 1 : 0;
+            r += x + 1 < m && less_entry(d4.y, i4.y, dj, ij) ? 1 : 0;
+            r += x + 2 < m && less_entry(d4.z, i4.z, dj, ij) ? 1 : 0;
+            r += x + 3 < m && less_entry(d4.w, i4.w, dj, ij) ? 1 : 0;
+        }
+        if (have) {
+            sd[r] = dj;
+            si[r] = ij;
+        }
+        const int q = have ? lower_bound_entries(pd, pi, size, dj, ij) + r : 0x7FFFFFFF;
+        const int low = __reduce_min_sync(kFull, q);
+        const int last = min(size + m, L) - 1;   // highest slot written
+        __syncwarp();
+        if (low > last) continue;
+        const int r_lo = low >> 5;
+        for (int row0 = last >> 5; row0 >= r_lo; row0 -= 4) {
+            float nd[4];
+            uint32_t ni[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int row = row0 - u;
+                if (row < r_lo) break;
+                const uint32_t taken = __reduce_or_sync(kFull, (q >> 5) == row ? 1u << (q & 31) : 0u);
+                const int before = __popc(__ballot_sync(kFull, q < 32 * row)) + __popc(taken & lt);
+                const int x = 32 * row + lane;
+                const bool cand = (taken >> lane) & 1u;
+                const float *ps = cand ? sd + before : pd + (x - before);
+                const uint32_t *pj = cand ? si + before : pi + (x - before);
+                nd[u] = *ps;
+                ni[u] = *pj;
+            }
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int x = 32 * (row0 - u) + lane;
+                if (row0 - u < r_lo) break;
+                if (x >= low && x <= last) {
+                    pd[x] = nd[u];
+                    pi[x] = ni[u];
+                }
+            }
+            __syncwarp();
+        }
+        size = last + 1;
+        cursor = min(cursor, low);
+    }
+    return size;
+}
 
 // Launch shape of a team of TW warps per query: CTAs of max(4, TW) warps,
 // with the register budget of min_blocks_per_sm<DT, NCH>() 4-warp CTAs per SM.
@@ -522,8 +623,9 @@ beam_search_kernel(const SearchArgs a) {
     static_assert(STG == 0 || TW == 1, "staging is for one-warp kernels");
     constexpr int S = STG;  // staged gather rows per buffer (0: registers)
     const size_t stage = S ? stage_bytes(DT, S, a.d >> 2) : 0;
-    unsigned char *tbase = smem_raw + (size_t)team * search_smem_per_team(lcap, hlog2, stage);
-    unsigned char *stg = tbase + search_smem_per_team(lcap, hlog2, 0);
+    unsigned char *tbase = smem_raw + (size_t)team * search_smem_per_team(a, stage);
+    unsigned char *stg = tbase + search_smem_per_team(a, 0);
+    constexpr int kCandCap = 32 * RPL;
     float *pd = reinterpret_cast<float *>(tbase);
     uint32_t *pi = reinterpret_cast<uint32_t *>(pd + lcap);
     float *cd = reinterpret_cast<float *>(pi + lcap);
@@ -532,6 +634,7 @@ beam_search_kernel(const SearchArgs a) {
     uint32_t *si = reinterpret_cast<uint32_t *>(sd + kCandCap);
     uint32_t *htab = si + kCandCap;
     volatile int *ctl = reinterpret_cast<volatile int *>(htab + H);  // claim, count, size
+    const CompactTable ct(reinterpret_cast<unsigned char *>(htab + H) + 16, a);   // used when a.ct_log2 != 0
 
     const int64_t slot = (int64_t)blockIdx.x * TPB + team;
     uint32_t *bits = a.vbits + slot * a.vbits_words;
@@ -649,9 +752,19 @@ beam_search_kernel(const SearchArgs a) {
         bool spilled = (H == 0), bad = false, overflow = false;
         if (leader) {
             for (int i = lane; i < H; i += 32) htab[i] = kNone;
+            if (a.ct_log2) {
+                ct.clear(lane);
+                spilled = false;
+            }
             __syncwarp();
+            bool to_bits = false;
+            if (a.ct_log2) {
+                ct.visit(a.entry, lane == 0, to_bits);
+                spilled = __any_sync(kFull, to_bits);   // (the entry itself, for the lines below)
+            }
             if (lane == 0) {
-                if (spilled) {
+                if (a.ct_log2 && !spilled) {
+                } else if (spilled) {
                     bitmap_visit(bits, a.entry);
                     vlog[0] = a.entry;
                 } else {
@@ -733,7 +846,7 @@ beam_search_kernel(const SearchArgs a) {
                 }
                 if (have_row) {
                     // Neighbour fetch + visited test-and-insert.
-                    if (!spilled && (int)(smem_count + rmax) > (H >> 1)) spilled = true;
+                    if (!a.ct_log2 && !spilled && (int)(smem_count + rmax) > (H >> 1)) spilled = true;
                     uint32_t nb[kMaxRowPerLane];
                     bool fresh[kMaxRowPerLane];
                     bool mybad = false;
@@ -756,6 +869,11 @@ beam_search_kernel(const SearchArgs a) {
                                 nbp[t] = (j < rmax) ? __ldg(a.adj + (size_t)pred_v * rmax + j) : kNone;
                             }
                         }
+                    } else if (!BI && sel2 >= 0) {
+                        // too few registers to hold it: ask L1 for that row (1 %)
+                        const char *r = reinterpret_cast<const char *>(a.adj + (size_t)(pi[sel2] & kIdMask) * rmax);
+                        const char *line = reinterpret_cast<const char *>(reinterpret_cast<uintptr_t>(r) & ~(uintptr_t)127) + 128 * lane;
+                        if (line < r + 4 * rmax) asm volatile("prefetch.global.L1 [%0];" ::"l"(line));
                     }
 #pragma unroll
                     for (int t = 0; t < kMaxRowPerLane; ++t) {
@@ -766,6 +884,7 @@ beam_search_kernel(const SearchArgs a) {
                             mybad = true;
                             continue;
                         }
+                        if (a.ct_log2) continue;
                         if (!spilled) {
                             fresh[t] = smem_visit(htab, hlog2, u, true) == 1;
                         } else if (H == 0 || smem_visit(htab, hlog2, u, false) == 2) {
@@ -773,6 +892,21 @@ beam_search_kernel(const SearchArgs a) {
                         }
                     }
                     if (__any_sync(kFull, mybad)) bad = true;
+                    if (a.ct_log2) {
+#pragma unroll
+                        for (int t = 0; t < kMaxRowPerLane; ++t) {
+                            const bool valid = (int64_t)nb[t] < a.n;   // (kNone is not)
+                            if (__ballot_sync(kFull, valid) == 0u) continue;
+                            bool to_bits = false;
+                            fresh[t] = ct.visit(nb[t], valid, to_bits);
+                            if (__any_sync(kFull, to_bits)) {
+                                if (to_bits) fresh[t] = bitmap_visit(bits, nb[t]);
+                                const unsigned m = __ballot_sync(kFull, to_bits && fresh[t]);
+                                if (to_bits && fresh[t]) vlog[nlog + __popc(m & ((1u << lane) - 1u))] = nb[t];
+                                nlog += __popc(m);
+                            }
+                        }
+                    }
 #pragma unroll
                     for (int t = 0; t < kMaxRowPerLane; ++t) {
                         const unsigned m = __ballot_sync(kFull, fresh[t]);
@@ -780,8 +914,16 @@ beam_search_kernel(const SearchArgs a) {
                         cnt += __popc(m);
                     }
                     __syncwarp();
-                    if (ROAR_PREFETCH_ROWS) prefetch_rows_l2(a.trav, (uint32_t)d * (4u >> DT), ci, cnt, lane);
-                    if (spilled) {  // every fresh id this hop went to the bitmap: log it
+                    if constexpr (DT == 0) {
+                        prefetch_rows_l2(a.trav, (uint32_t)d * 4u, ci, cnt, lane);
+                    } else {
+#pragma unroll
+                        for (int t = 0; t < kMaxRowPerLane; ++t)
+                            if (fresh[t]) prefetch_row_l2(a.trav, (uint32_t)d * (4u >> DT), nb[t]);
+                    }
+                    if (a.ct_log2) {
+                        // ids that went to the bitmap are logged above
+                    } else if (spilled) {  // every fresh id this hop went to the bitmap: log it
                         for (int j = lane; j < cnt; j += 32) vlog[nlog + j] = ci[j];
                         nlog += cnt;
                     } else {
@@ -841,77 +983,7 @@ beam_search_kernel(const SearchArgs a) {
                 __syncwarp();
                 if (cnt == 0) continue;
             }
-            // Sort the candidates (ids are distinct, so ranks are a permutation).
-#pragma unroll
-            for (int t = 0; t < kMaxCandPerLane; ++t) {
-                const int j = lane + 32 * t;
-                if (j < cnt) {
-                    const float dj = cd[j];
-                    const uint32_t ij = ci[j];
-                    int r = 0;
-                    for (int x = 0; x < cnt; ++x) r += less_entry(cd[x], ci[x], dj, ij) ? 1 : 0;
-                    sd[r] = dj;
-                    si[r] = ij;
-                }
-            }
-            __syncwarp();
-            // Final slot of sorted candidate r: (#pool entries before it) + r.
-            int cpos[kMaxCandPerLane];
-#pragma unroll
-            for (int t = 0; t < kMaxCandPerLane; ++t) {
-                const int r = lane + 32 * t;
-                cpos[t] = r < cnt ? lower_bound_entries(pd, pi, size, sd[r], si[r]) + r : 0x7FFFFFFF;
-            }
-            const int pmin = __shfl_sync(kFull, cpos[0], 0);
-            if (cnt <= 4) {
-                // Few candidates (the usual case once the pool is full): insert
-                // them one at a time in increasing slot order. (A single
-                // destination-driven pass for all of them measured 1-2 % slower
-                // on GB300: its scalar shared-memory reads conflict on banks.)
-                int sz = size;
-                for (int r = 0; r < cnt; ++r) {
-                    const int pos = __shfl_sync(kFull, cpos[0], r);
-                    if (pos >= L) break;
-                    pool_insert_one(pd, pi, sz, L, pos, sd[r], si[r], lane);
-                    sz = min(L, sz + 1);
-                }
-                size = sz;
-                cursor = min(cursor, pmin);
-                __syncwarp();
-                continue;
-            }
-            // Many candidates: move the pool tail [pmin, size) up in place, 32
-            // entries at a time from the end: new slots are increasing and never
-            // below the old ones, so no write lands on an entry not yet read.
-            for (int hi = size; hi > pmin; hi -= 32) {
-                const int i = hi - 32 + lane;
-                const bool act = i >= pmin;
-                float di = 0.f;
-                uint32_t ii = 0;
-                int np = 0;
-                if (act) {
-                    di = pd[i];
-                    ii = pi[i];
-                    np = i + lower_bound_entries(sd, si, cnt, di, ii & kIdMask);
-                }
-                __syncwarp();
-                if (act && np < L) {
-                    pd[np] = di;
-                    pi[np] = ii;
-                }
-                __syncwarp();
-            }
-#pragma unroll
-            for (int t = 0; t < kMaxCandPerLane; ++t) {
-                const int r = lane + 32 * t;
-                if (r < cnt && cpos[t] < L) {
-                    pd[cpos[t]] = sd[r];
-                    pi[cpos[t]] = si[r];
-                }
-            }
-            size = min(L, size + cnt);
-            cursor = min(cursor, pmin);
-            __syncwarp();
+            size = pool_merge(pd, pi, size, L, cd, ci, cnt, sd, si, cursor, lane);
         }
 
         // Output (re-ranked in FP32, in place, for the reduced-precision forms).
@@ -1020,7 +1092,7 @@ const void *kernel_table(int nch, int rpl, int tw, bool staged) {
 #define ROAR_K(N, R, T) \
     if (nch == N && rpl == R && tw == T && !staged) return (const void *)beam_search_kernel<DT, N, R, T, 0>;
 #define ROAR_KS(N, R)                                                                              \
-    if constexpr (stage_rows(DT, N) > 0) {                                                         \
+    if constexpr (N == 2 && stage_rows(DT, N) > 0) {                                               \
         if (nch == N && rpl == R && tw == 1 && staged)                                             \
             return (const void *)beam_search_kernel<DT, N, R, 1, stage_rows(DT, N)>;               \
     }

@@ -1,0 +1,80 @@
+"""The compact visited table and the pool merge of the search kernels, where they can go wrong: rows that repeat an id,
+ids whose slot value is the free mark, tables that overflow into the bitmap, tiny sets, wide graph rows, and every team
+size and batch size the launch rules tell apart. Everything equals the oracle's search."""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_util import assert_same, dev_index, run
+
+pytestmark = pytest.mark.gpu
+
+
+def _graph(rng, n, r, special=None):
+    adj = rng.integers(0, n, (n, r)).astype(np.uint32)
+    adj[:, 1::5] = adj[:, 0::5][:, :adj[:, 1::5].shape[1]]           # the same id twice in a row
+    if special is not None:
+        adj[rng.random((n, r)) < 0.05] = rng.choice(special)
+    pad = rng.integers(r // 2, r + 1, n)
+    adj[np.arange(r)[None, :] >= pad[:, None]] = 0xFFFFFFFF
+    return adj
+
+
+def _unit(rng, n, d):
+    x = rng.standard_normal((n, d)).astype(np.float32)
+    return x / np.linalg.norm(x, axis=1, keepdims=True)
+
+
+@pytest.mark.parametrize("n,d,r,L,k,nq", [
+    (33, 8, 8, 10, 5, 3), (100, 16, 64, 100, 10, 40), (5000, 64, 64, 3, 1, 200), (5000, 64, 96, 33, 10, 50),
+    (5000, 132, 128, 128, 100, 20), (20_000, 200, 33, 31, 10, 700), (20_000, 40, 70, 500, 10, 30),
+    (3000, 300, 48, 1024, 100, 8)])
+def test_sizes_teams_and_repeated_ids(n, d, r, L, k, nq):
+    rng = np.random.default_rng(n + L)
+    X, Q, adj = _unit(rng, n, d), _unit(rng, nq, d), _graph(rng, n, r)
+    ref = oracle.beam_search(X, adj, 0, Q, k, L, max_visits=16384)
+    idx = dev_index(X, adj, 0)
+    assert_same(run(idx, Q, k, L), ref, "automatic")
+    for tw, hash_log2 in ((1, 0), (2, 0), (4, -1), (8, 0), (1, 10)):
+        idx.set_tuning(L, tw, hash_log2)
+        assert_same(run(idx, Q, k, L), ref, f"team {tw} table {hash_log2}")
+    idx.close()
+
+
+def test_values_that_equal_the_free_mark():
+    # 23-bit ids over 2^7 buckets: 16 bits in a slot, so 0xFFFF is a possible value; the entry and many neighbours have it
+    n, L = 5_000_000, 10
+    u = np.arange(n, dtype=np.uint64)
+    h = (u * 2654435769) & ((1 << 23) - 1)
+    special = u[(h & 0xFFFF) == 0xFFFF].astype(np.uint32)
+    assert len(special) > 20
+    rng = np.random.default_rng(1)
+    X, Q = _unit(rng, n, 4), _unit(rng, 300, 4)
+    adj = _graph(rng, n, 8, special)
+    ref = oracle.beam_search(X, adj, int(special[0]), Q, 5, L, max_visits=16384)
+    idx = dev_index(X, adj, int(special[0]))
+    assert_same(run(idx, Q, 5, L), ref)
+    assert_same(run(idx, Q, 5, L), ref, "bitmap clean after the first batch")
+    idx.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "fp8"])
+@pytest.mark.parametrize("cap", [16384, 900])
+def test_full_buckets_go_to_the_bitmap(dtype, cap):
+    # a full grid of wide searches: few slots per query for many visits (and a visit cap that ends them in the middle)
+    n, d, L, nq = 300_000, 16, 400, 5000
+    rng = np.random.default_rng(2)
+    X, Q, adj = _unit(rng, n, d), _unit(rng, nq, d), _graph(rng, n, 64)
+    codes = scales = None
+    if dtype == "bf16":
+        codes = oracle.quant_bf16(X)
+    elif dtype == "fp8":
+        codes, scales = oracle.quant_e4m3(X)
+    kw = {} if dtype == "f32" else {"dtype": dtype, "Xt": codes, "scales": scales}
+    ref = oracle.beam_search(X, adj, 7, Q[:48], 10, L, max_visits=cap, **kw)
+    idx = dev_index(X, adj, 7, dtype=dtype, trav=codes.view(np.int16) if dtype == "bf16" else codes, scales=scales,
+                    max_visits=cap)
+    for again in range(2):
+        got = run(idx, Q, 10, L)
+        assert_same([g[:48] for g in got], ref, f"pass {again}")
+    idx.close()

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <numeric>
@@ -57,14 +58,22 @@ struct roar_index {
     // warps per query team, visited-table mode (0 auto, -1 bitmap only,
     // 5..15 shared slots log2), resident-CTA cap per SM (0 = occupancy limit).
     struct Tune {
-        int tw = 1;
+        int tw = 0;     // 0: by the number of queries (team_for)
         int hash = 0;
         int bps_cap = 0;
     } tune[6];
-    // scratch: one visited bitmap + log per resident warp, grown on demand
-    uint32_t *vbits = nullptr;
-    uint32_t *vlog = nullptr;
-    int64_t vslots = 0;
+    // scratch: one visited bitmap + log per resident warp, replaced by a larger
+    // one on demand; captured plans and servers hold the one they point at
+    struct Scratch {
+        uint32_t *vbits = nullptr;
+        uint32_t *vlog = nullptr;
+        int64_t slots = 0;
+        ~Scratch() {
+            cudaFree(vbits);
+            cudaFree(vlog);
+        }
+    };
+    std::shared_ptr<Scratch> scratch;
     int64_t vbits_words = 0;
     int32_t vlog_cap = 0;
     unsigned int *work = nullptr;
@@ -202,8 +211,6 @@ extern "C" roar_status roar_index_set_tombstones(roar_index *idx, const uint32_t
 extern "C" void roar_index_destroy(roar_index *idx) {
     if (!idx) return;
     cudaDeviceSynchronize();
-    cudaFree(idx->vbits);
-    cudaFree(idx->vlog);
     cudaFree(idx->work);
     cudaFree(idx->stage);
     delete idx;
@@ -213,36 +220,48 @@ namespace roar {
 
 // Make room for `slots` visited bitmaps and logs (synchronises the device when it grows).
 static roar_status ensure_scratch(roar_index *idx, int64_t slots) {
-    if (slots <= idx->vslots) return ROAR_OK;
+    if (idx->scratch && slots <= idx->scratch->slots) return ROAR_OK;
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(e, "ensure_scratch");
-    cudaFree(idx->vbits);
-    cudaFree(idx->vlog);
-    idx->vbits = nullptr;
-    idx->vlog = nullptr;
-    idx->vslots = 0;
+    idx->scratch.reset();   // freed here unless a plan or a server still uses it
+    std::shared_ptr<roar_index::Scratch> n(new (std::nothrow) roar_index::Scratch());
+    if (!n) return ROAR_ENOMEM;
     const size_t bb = (size_t)slots * idx->vbits_words * sizeof(uint32_t);
-    e = cudaMalloc(&idx->vbits, bb);
-    if (e == cudaSuccess) e = cudaMalloc(&idx->vlog, (size_t)slots * idx->vlog_cap * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMemset(idx->vbits, 0, bb);
+    e = cudaMalloc(&n->vbits, bb);
+    if (e == cudaSuccess) e = cudaMalloc(&n->vlog, (size_t)slots * idx->vlog_cap * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMemset(n->vbits, 0, bb);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
-        cudaFree(idx->vbits);
-        cudaFree(idx->vlog);
-        idx->vbits = nullptr;
-        idx->vlog = nullptr;
         cudaGetLastError();
         set_error("roar_search: cannot allocate the visited bitmaps");
         return ROAR_ENOMEM;
     }
-    idx->vslots = slots;
+    n->slots = slots;
+    idx->scratch = n;
     return ROAR_OK;
 }
+
+std::shared_ptr<void> hold_scratch(const roar_index *idx) { return idx->scratch; }
 
 int tune_bucket(int L) {
     int b = 0;
     while (b < 5 && (32 << b) < L) ++b;
     return b;
+}
+
+// Warps per query of an untuned launch: the widest team with which all nq
+// queries are resident at once (more queries run one warp each). Measured on
+// GB300, 1M x 200 FP32, L = 100, teams of 1 / 2 / 4 / 8 warps: 1 query 854 / 711 /
+// 623 / 585 us, 300 queries 1348 / 1073 / 934 / 868, 600 queries 1402 / 1123 /
+// 981 / 1333, 1,200 queries 1447 / 1165 / 1535 / 2259, 2,400 queries 1885 / 2058 /
+// 2669 / 4217.
+static int team_for(const SearchArgs &a, int64_t nq, int sms) {
+    if (a.bi_off) return 1;
+    for (int tw = 8; tw > 1; tw /= 2) {
+        if (nq > (int64_t)sms * kMaxWarpsPerSm / tw) continue;
+        if (nq <= (int64_t)search_blocks_per_sm(a, tw) * teams_per_block(tw) * sms) return tw;
+    }
+    return 1;
 }
 
 // Fill a SearchArgs for the handle and pick the launch shape.
@@ -266,10 +285,11 @@ roar_status plan_search(roar_index *idx, int32_t lmax, SearchArgs &a, int &block
     a.bi_nt = idx->bi_nt;
     const bool bi = idx->bi_off != nullptr;
     tw = t.tw;
-    if (bi && tw != 1) {
+    if (bi && tw > 1) {
         set_error("roar_search: the bipartite-graph search runs one warp per query");
         return ROAR_EINVAL;
     }
+    if (tw == 0) tw = team_for(a, nq, idx->num_sms);
     choose_visited(a, t.hash, tw, lmax, nq, idx->num_sms);
     int bps = search_blocks_per_sm(a, tw);
     if (bps <= 0) {
@@ -283,9 +303,9 @@ roar_status plan_search(roar_index *idx, int32_t lmax, SearchArgs &a, int &block
     blocks = (int)std::max<int64_t>(1, std::min(want, full));
     roar_status st = ensure_scratch(idx, full * tpb);
     if (st != ROAR_OK) return st;
-    a.vbits = idx->vbits;
+    a.vbits = idx->scratch->vbits;
     a.vbits_words = idx->vbits_words;
-    a.vlog = idx->vlog;
+    a.vlog = idx->scratch->vlog;
     a.vlog_cap = idx->vlog_cap;
     a.work = idx->work;
     return ROAR_OK;
@@ -443,6 +463,7 @@ struct roar_plan {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int32_t *order = nullptr;  // owned processing order (longest beam first), or null
+    std::shared_ptr<void> scratch;   // the visited scratch the captured launch points at
 };
 
 extern "C" roar_status roar_plan_create(roar_index *idx, const float *queries, int64_t nq,
@@ -493,6 +514,7 @@ extern "C" roar_status roar_plan_create(roar_index *idx, const float *queries, i
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&p->exec, p->graph, 0);
         if (cs) cudaStreamDestroy(cs);
+        p->scratch = hold_scratch(idx);
         if (e != cudaSuccess) st = cuda_fail(e, "roar_plan_create: capture");
     }
     if (st != ROAR_OK) {

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
+
 #include "roargraph.h"
 
 namespace roar {
@@ -192,5 +194,9 @@ void choose_visited(SearchArgs &a, int hash, int tw, int L, int64_t nq, int sms)
 // Fills a SearchArgs for a handle (index rows, tuning, scratch sized for the
 // full resident grid) and picks blocks and team warps. Defined in roar_capi.cu.
 roar_status plan_search(roar_index *idx, int32_t lmax, SearchArgs &a, int &blocks, int &tw, int64_t nq);
+// Keeps the visited scratch the handle's last plan_search pointed at alive: a
+// later, larger search replaces the handle's, but not that of a captured plan or
+// a server. (The caller holds the handle's lock or is its only user.)
+std::shared_ptr<void> hold_scratch(const roar_index *idx);
 
 }  // namespace roar

@@ -80,6 +80,7 @@ cudaError_t host_pinned(T **h, size_t count) {
 
 struct roar_server {
     roar_index *idx = nullptr;
+    std::shared_ptr<void> scratch;   // the visited scratch the kernel's arguments point at
     int32_t d = 0, k_max = 0, L_max = 0, tw = 1;
     int64_t R = 0;
     uint32_t idle_polls = 50000;
@@ -273,6 +274,7 @@ extern "C" roar_status roar_server_create(roar_index *idx, const roar_server_cfg
         delete s;
         return st;
     }
+    s->scratch = hold_scratch(idx);
     s->d = a.d;
     // Ring capacity: given, or as many k_max-wide slots as the budget could
     // hold; the budget itself is enforced per request at submission.

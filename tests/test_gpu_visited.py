@@ -78,3 +78,28 @@ def test_full_buckets_go_to_the_bitmap(dtype, cap):
         got = run(idx, Q, 10, L)
         assert_same([g[:48] for g in got], ref, f"pass {again}")
     idx.close()
+
+
+def test_a_plan_outlives_the_scratch_it_was_captured_with():
+    # a small captured batch (wide teams, few scratch slots), then a batch that needs more scratch, then the plan again
+    import torch
+
+    n, d, r = 20_000, 32, 32
+    rng = np.random.default_rng(6)
+    X, Q, adj = _unit(rng, n, d), _unit(rng, 4000, d), _graph(rng, n, r)
+    k = np.full(20, 10, np.int32)
+    L = np.arange(60, 80).astype(np.int32)
+    idx = dev_index(X, adj, 3)
+    out = idx.uneven_outputs(k)
+    plan = idx.plan_uneven(torch.from_numpy(Q[:20]).to("cuda:0"), torch.from_numpy(k).to("cuda:0"),
+                           torch.from_numpy(L).to("cuda:0"), 80, out)
+    assert_same(run(idx, Q, 5, 10), oracle.beam_search(X, adj, 3, Q, 5, 10, max_visits=16384), "large batch")
+    for _ in range(2):
+        plan.launch()
+        torch.cuda.synchronize()
+        ids = out[1].cpu().numpy().view(np.uint32).reshape(20, 10)
+        for i in range(20):
+            ref = oracle.beam_search(X, adj, 3, Q[i:i + 1], 10, int(L[i]), max_visits=16384)
+            assert np.array_equal(ids[i], ref[0][0]), i
+    plan.close()
+    idx.close()

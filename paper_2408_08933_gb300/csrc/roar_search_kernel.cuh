@@ -243,6 +243,14 @@ __device__ __forceinline__ float reduce_rows(const float (&s)[B], int lane) {
     return v[0];
 }
 
+// The two FP32 halves of s: fmaf(q, x, low), fmaf(q, y, high).
+__device__ __forceinline__ void fma_pair(unsigned long long &s, float q, float x, float y) {
+    unsigned long long q2, x2;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(q2) : "f"(q));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x2) : "f"(x), "f"(y));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(s) : "l"(q2), "l"(x2));
+}
+
 // Distances for rows ids_s[j] (shared, expanded bit ignored), j = first,
 // first + 1, ... in groups of B, groups `step` apart (one warp's share of a
 // team); writes -<q, x> (times the row scale for FP8) to out_s[j].
@@ -282,18 +290,40 @@ __device__ __forceinline__ void score_rows(const void *base, const float *scales
             }
         }
         float s[B];
+        if constexpr (DT == 2 && B % 2 == 0) {
+            // Two rows per instruction, each with its own sum in the fixed order.
+            // (FP8, L = 100: 4.85 -> 4.66 ms; BF16 was 8 % slower, and FP32 rows
+            // would have to be interleaved first.)
 #pragma unroll
-        for (int b = 0; b < B; ++b) {
-            s[b] = 0.0f;
+            for (int b = 0; b < B; b += 2) {
+                unsigned long long s2 = 0ull;
 #pragma unroll
-            for (int c = 0; c < NCH; ++c) {
-                const int ch = lane + 32 * c;
-                if (ch < d4) {
-                    const float4 x = to_f4<DT>(raw[b][c]);
-                    s[b] = fmaf(qr[c].x, x.x, s[b]);
-                    s[b] = fmaf(qr[c].y, x.y, s[b]);
-                    s[b] = fmaf(qr[c].z, x.z, s[b]);
-                    s[b] = fmaf(qr[c].w, x.w, s[b]);
+                for (int c = 0; c < NCH; ++c) {
+                    const int ch = lane + 32 * c;
+                    if (ch < d4) {
+                        const float4 x = to_f4<DT>(raw[b][c]), y = to_f4<DT>(raw[b + 1][c]);
+                        fma_pair(s2, qr[c].x, x.x, y.x);
+                        fma_pair(s2, qr[c].y, x.y, y.y);
+                        fma_pair(s2, qr[c].z, x.z, y.z);
+                        fma_pair(s2, qr[c].w, x.w, y.w);
+                    }
+                }
+                asm("mov.b64 {%0, %1}, %2;" : "=f"(s[b]), "=f"(s[b + 1]) : "l"(s2));
+            }
+        } else {
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                s[b] = 0.0f;
+#pragma unroll
+                for (int c = 0; c < NCH; ++c) {
+                    const int ch = lane + 32 * c;
+                    if (ch < d4) {
+                        const float4 x = to_f4<DT>(raw[b][c]);
+                        s[b] = fmaf(qr[c].x, x.x, s[b]);
+                        s[b] = fmaf(qr[c].y, x.y, s[b]);
+                        s[b] = fmaf(qr[c].z, x.z, s[b]);
+                        s[b] = fmaf(qr[c].w, x.w, s[b]);
+                    }
                 }
             }
         }

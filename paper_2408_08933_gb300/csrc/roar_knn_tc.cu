@@ -57,7 +57,8 @@ constexpr int kC = 128;            // candidates kept per row
 constexpr int kMaxStages = 16;
 constexpr int kCols = 128;         // columns of a tile one epilogue warp filters
 constexpr int kTrimMost = 384;     // entries of a row a trim takes in registers (12 per lane)
-constexpr int kSegCap = kTrimMost + kCols;   // entries of one segment of a row's candidate buffer
+constexpr int kSegCut = 256;       // a segment of a row's candidate buffer with more entries is cut at once;
+constexpr int kSegCap = kSegCut + kCols;     // so that it can take another tile's
 constexpr uint64_t kDrainNs = 2000000000ull;  // bound of the final wait for issued MMAs and copies
 constexpr int kTmemCols = 512;     // 2 accumulators of 256 columns
 constexpr uint32_t kChunkA = kTM * kKC * 2;   // 16 KB: one CTA's T rows, a 64-wide K chunk
@@ -785,6 +786,20 @@ knn_tc_kernel(const KnnUnits u, int stages, uint2 *__restrict__ scratch, uint2 *
                     !__all_sync(kFull, mbar_wait(&acc_full[set], (acc >> 1) & 1, abort_v, wait_ns)))
                     dead = true;
                 if (mine && !dead) {
+                    uint32_t full = __ballot_sync(kFull, cnt > kSegCut);
+                    while (full) {   // filled before its trim is due, or left so by ties
+                        const int src = __ffs(full) - 1;
+                        full &= full - 1;
+                        RowList<1> one;
+                        one.base = wbuf + (int64_t)(src * kSegs + seg) * kSegCap;
+                        one.m[0] = __shfl_sync(kFull, cnt, src);
+                        const float th = warp_cut<kSegCap / 32>(one, kC, lane, [&](int i, uint2 v) { one.base[i] = v; });
+                        if (lane == src) {
+                            thr = fmaxf(thr, th);
+                            cnt = kC;
+                            end = mybuf + 8 * kC;
+                        }
+                    }
                     tc_fence_after();
 #pragma unroll 1
                     for (int c = 0; c < kCols; c += 64) {
@@ -802,20 +817,6 @@ knn_tc_kernel(const KnnUnits u, int stages, uint2 *__restrict__ scratch, uint2 *
                     }
                     cnt = (int)((end - mybuf) >> 3);
                     __syncwarp();
-                    uint32_t full = __ballot_sync(kFull, cnt > kSegCap - kCols);
-                    while (full) {   // a segment that filled before its trim is due
-                        const int src = __ffs(full) - 1;
-                        full &= full - 1;
-                        RowList<1> one;
-                        one.base = wbuf + (int64_t)(src * kSegs + seg) * kSegCap;
-                        one.m[0] = __shfl_sync(kFull, cnt, src);
-                        const float th = warp_cut<kSegCap / 32>(one, kC, lane, [&](int i, uint2 v) { one.base[i] = v; });
-                        if (lane == src) {
-                            thr = fmaxf(thr, th);
-                            cnt = kC;
-                            end = mybuf + 8 * kC;
-                        }
-                    }
                 }
                 // Trim the lists each time the rows of X seen have doubled
                 // (about kC new entries per row each).

@@ -168,12 +168,13 @@ __host__ __device__ inline bool search_staged(int dtype, int d, int tw, int lcap
            ((size_t)d * (4 >> dtype)) % 16 == 0;
 }
 
+constexpr int kCtlBytes = 32;
 // Shared memory of one team: pool (8 B per slot), candidate buffers (16 B per
-// slot), optional visited table (4 B per slot), a 16-byte control block
-// (claimed query, hop count, pool size), optional compact visited table, then
+// slot), optional visited table (4 B per slot), a control block (claimed query,
+// hop count, pool size, next node), optional compact visited table, then
 // `stage` bytes of gather staging.
 __host__ __device__ inline size_t search_smem_per_team(const SearchArgs &a, size_t stage) {
-    return (size_t)a.lcap * 8 + (size_t)cand_cap(a.rmax) * 16 + (a.hash_log2 ? ((size_t)4 << a.hash_log2) : 0) + 16 +
+    return (size_t)a.lcap * 8 + (size_t)cand_cap(a.rmax) * 16 + (a.hash_log2 ? ((size_t)4 << a.hash_log2) : 0) + kCtlBytes +
            ct_bytes(a.ct_log2) + stage;
 }
 // Resident CTAs per SM for this launch with teams of tw warps (0 if it

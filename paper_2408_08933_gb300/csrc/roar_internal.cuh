@@ -37,6 +37,12 @@ constexpr int kMinBlocksPerSm = ROAR_MIN_BLOCKS;  // register budget: 65536 / (b
 #ifndef ROAR_MIN_BLOCKS_LOWP_WIDE
 #define ROAR_MIN_BLOCKS_LOWP_WIDE 4
 #endif
+// One-warp BF16 searches of 257 to 512 columns, with no spills: 3 CTAs per SM, with 4
+// rows per batch (d = 512, L = 100 6.70 ms, 4 CTAs 7.01, 5 CTAs 7.15; FP8 the other
+// way round, 7.38 and 6.25).
+#ifndef ROAR_MIN_BLOCKS_BF16_512
+#define ROAR_MIN_BLOCKS_BF16_512 3
+#endif
 template <int DT, int NCH = 1>
 __host__ __device__ constexpr int min_blocks_per_sm() {
     return DT == 0 ? ROAR_MIN_BLOCKS

@@ -331,9 +331,11 @@ def _serve_rate(srv, Qpool, rate, duration, seed_tag):
             "unfinished_requests": int(n - len(lats))}
 
 
-def _traffic(kernel_file, src_hash):
+def _traffic(kernel_file, src_hash, key="traffic_bytes_per_launch"):
     """ncu DRAM bytes per launch from the committed profile summary, if it
-    was taken on the current kernel source; else None."""
+    was taken on the current kernel source; else None. The FP32 summary has two
+    launches: the bitmap alone as visited set (the default key) and the
+    automatic one (key + "_auto")."""
     p = os.path.join(ROOT, "profiles", kernel_file)
     if not os.path.exists(p):
         return None
@@ -345,7 +347,7 @@ def _traffic(kernel_file, src_hash):
     if vals.get("kernel_source_sha") != src_hash:
         return None
     try:
-        return float(vals["traffic_bytes_per_launch"])
+        return float(vals[key])
     except (KeyError, ValueError):
         return None
 
@@ -867,7 +869,9 @@ def main():
                           "paper_2408_08933_gb300/csrc/roar_search.cu",
                           "paper_2408_08933_gb300/csrc/roar_internal.cuh",
                           "paper_2408_08933_gb300/csrc/roar_search_f32.cu"])
-    traffic = _traffic(f"search_f32_{w.name}.txt", src_hash)
+    # The DRAM bytes of the launch that was timed: its visited set decides which.
+    key = {0: "traffic_bytes_per_launch_auto", 1: "traffic_bytes_per_launch"}.get(best % 4 if best >= 0 else 0)
+    traffic = _traffic(f"search_f32_{w.name}.txt", src_hash, key) if key else None
 
     # ---- e2e: host buffers through roar_search_host -----------------------------
     Qh = torch.from_numpy(Q).pin_memory()

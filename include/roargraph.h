@@ -165,10 +165,10 @@ void roar_index_destroy(roar_index *idx);
 
 /*
  * Tuning: shared-memory visited-table capacity 2^log2 slots per query
- * (5 <= log2 <= 15), 0 to choose from L automatically, or -1 for no shared
- * table. A query that visits more than half the table continues in its exact
- * global visited bitmap, so results never depend on this setting; speed and
- * occupancy do.
+ * (5 <= log2 <= 15), 0 to choose automatically (a compact exact table of 16-bit
+ * slots where it pays), or -1 for no shared table. What a table cannot take
+ * continues in the query's exact global visited bitmap, so results never depend
+ * on this setting; speed and occupancy do.
  * Errors: ROAR_EINVAL.
  */
 roar_status roar_index_set_hash_log2(roar_index *idx, int32_t log2);
@@ -266,7 +266,8 @@ void roar_plan_destroy(roar_plan *plan);
  * Launch tuning for the beam-width bucket that contains L (L <= 32, 64, 128,
  * 256, 512, 1024): team_warps in {1, 2, 4, 8} warps per query (32..256
  * threads), hash_log2 as in roar_index_set_hash_log2, blocks_per_sm_cap = 0
- * for the occupancy limit. Results never depend on the tuning.
+ * for the occupancy limit. Untuned, a launch takes the widest team with which
+ * all its queries are resident at once. Results never depend on the tuning.
  * Errors: ROAR_EINVAL.
  */
 roar_status roar_index_set_tuning(roar_index *idx, int32_t L, int32_t team_warps, int32_t hash_log2,
@@ -406,9 +407,10 @@ roar_status roar_quantize(const float *X, int64_t n, int32_t d, roar_dtype dtype
  *   kk                    1..128, kk <= n.
  *   ids, dist             device [nt][kk] outputs.
  * Allocates and frees its own device scratch (BF16 copies of T and X with
- * rows padded to a multiple of 64 columns, and candidate buffers of 8 KB per
- * query row for up to 131,072 rows at a time)
- * and synchronises `stream` before returning. Errors: ROAR_EINVAL,
+ * rows padded to a multiple of 16 columns, candidate buffers of 3 MB per CTA
+ * pair, candidate lists) and synchronises `stream` before returning; scratch of
+ * up to 320 MB in all comes from a pool that keeps at most that much per device
+ * between calls. Errors: ROAR_EINVAL,
  * ROAR_ENOMEM, ROAR_ECUDA, ROAR_ETIMEOUT (a bounded tensor-core wait gave up).
  */
 roar_status roar_knn(const float *T, int64_t nt, const float *X, int64_t n, int32_t d, int32_t kk,

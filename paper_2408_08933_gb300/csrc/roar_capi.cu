@@ -301,7 +301,12 @@ roar_status plan_search(roar_index *idx, int32_t lmax, SearchArgs &a, int &block
     int64_t want = (nq + tpb - 1) / tpb;
     int64_t full = (int64_t)bps * idx->num_sms;
     blocks = (int)std::max<int64_t>(1, std::min(want, full));
-    roar_status st = ensure_scratch(idx, full * tpb);
+    // Scratch for the widest launch at this L, not only for this one: a warm-up
+    // of a few queries (wide teams, few slots) is enough before a capture of many.
+    SearchArgs one = a;
+    one.hash_log2 = one.ct_log2 = one.staged = 0;
+    const int64_t widest = (int64_t)search_blocks_per_sm(one, 1) * teams_per_block(1) * idx->num_sms;
+    roar_status st = ensure_scratch(idx, std::max(full * tpb, widest));
     if (st != ROAR_OK) return st;
     a.vbits = idx->scratch->vbits;
     a.vbits_words = idx->vbits_words;

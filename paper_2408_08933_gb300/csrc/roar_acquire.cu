@@ -258,7 +258,7 @@ acquire_kernel(const float *__restrict__ X, int64_t n, int d, const uint32_t *__
                 if (!all || nr == M) break;
                 const int f = __ffs(all) - 1;   // the nearest survivor is kept
                 if (f / G == w) {
-if (nr < scap) {
+                    if (nr < scap) {
 #pragma unroll
                         for (int c = 0; c < NCH; ++c) {
                             // picked by masks: selects made the compiler index qc in local memory
@@ -271,7 +271,7 @@ if (nr < scap) {
                                 v.z |= __float_as_uint(qc[g][c].z) & m;
                                 v.w |= __float_as_uint(qc[g][c].w) & m;
                             }
-                            if (lane + 32 * c < d4) 
+                            if (lane + 32 * c < d4)
                                 reinterpret_cast<uint4 *>(rows)[(size_t)nr * d4 + lane + 32 * c] = v;
                         }
                     }

@@ -13,6 +13,7 @@
 #include "roar_internal.cuh"
 
 namespace roar {
+void knn_pool_trim();
 
 static thread_local char g_last_error[256] = "";
 
@@ -214,6 +215,7 @@ extern "C" void roar_index_destroy(roar_index *idx) {
     cudaFree(idx->work);
     cudaFree(idx->stage);
     delete idx;
+    knn_pool_trim();
 }
 
 namespace roar {

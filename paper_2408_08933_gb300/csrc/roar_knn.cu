@@ -275,15 +275,15 @@ namespace roar {
 // cudaMalloc (10,000 x 1M x 200: 7.24 ms from the pool, 7.05 ms without).
 constexpr uint64_t kKnnPoolKeep = 320ull << 20;   // a full grid's candidate buffers (239 MB) and small operands
 constexpr int kMaxDevices = 128;
+static std::mutex g_knn_pool_mu;
+static cudaMemPool_t g_knn_pools[kMaxDevices] = {};
 static cudaError_t knn_pool(cudaMemPool_t *pool) {
-    static std::mutex mu;
-    static cudaMemPool_t pools[kMaxDevices] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!pools[dev]) {
+    std::lock_guard<std::mutex> lock(g_knn_pool_mu);
+    if (!g_knn_pools[dev]) {
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
@@ -296,10 +296,16 @@ static cudaError_t knn_pool(cudaMemPool_t *pool) {
             if (p) cudaMemPoolDestroy(p);
             return e;
         }
-        pools[dev] = p;
+        g_knn_pools[dev] = p;
     }
-    *pool = pools[dev];
+    *pool = g_knn_pools[dev];
     return cudaSuccess;
+}
+// Gives back what the pools hold and no call is using.
+void knn_pool_trim() {
+    std::lock_guard<std::mutex> lock(g_knn_pool_mu);
+    for (cudaMemPool_t p : g_knn_pools)
+        if (p) cudaMemPoolTrimTo(p, 0);
 }
 }  // namespace roar
 

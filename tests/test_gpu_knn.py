@@ -72,3 +72,19 @@ def test_knn_sorted_rows(reverse):
     want = np.arange(10) if reverse else n - 1 - np.arange(10)
     for r in range(0, 200, 9):
         assert set(ids[r].tolist()) == set(want.tolist())
+
+
+def test_a_destroyed_index_gives_the_pool_back():
+    import torch
+    from gpu_util import dev_index
+
+    rng = np.random.default_rng(6)
+    X = rng.standard_normal((10_000, 64)).astype(np.float32)
+    T = rng.standard_normal((1000, 64)).astype(np.float32)
+    first = _knn(T, X, 50)
+    held = torch.cuda.mem_get_info()[0]
+    dev_index(X[:100], np.full((100, 8), 0xFFFFFFFF, np.uint32), 0).close()
+    # the least a call holds: candidate buffers of 3 MB per pair, at least one pair per 256 T rows
+    assert torch.cuda.mem_get_info()[0] - held >= 4 * 3 << 20
+    again = _knn(T, X, 50)
+    assert np.array_equal(first[0], again[0]) and np.array_equal(first[1], again[1])

@@ -126,3 +126,28 @@ def test_a_small_warm_up_is_enough_before_a_capture():
     got = (got[0].view(np.uint32), got[1], got[2].view(np.uint32), got[3].view(np.uint32), got[4])
     assert_same(got, oracle.beam_search(X, adj, 3, Q, 10, 40, max_visits=16384))
     idx.close()
+
+
+def test_a_small_warm_up_is_enough_for_the_staged_gather():
+    # the bitmap alone at 129 to 256 columns: the large launch stages its gathers, with more CTAs per SM
+    import torch
+
+    n, d, r, nq = 20_000, 200, 32, 4000
+    rng = np.random.default_rng(9)
+    X, Q, adj = _unit(rng, n, d), _unit(rng, nq, d), _graph(rng, n, r)
+    idx = dev_index(X, adj, 3)
+    idx.set_hash_log2(-1)
+    q = torch.from_numpy(Q).to("cuda:0")
+    out = (torch.empty((nq, 10), dtype=torch.int32, device="cuda:0"), torch.empty((nq, 10), device="cuda:0"),
+           *(torch.empty(nq, dtype=torch.int32, device="cuda:0") for _ in range(3)))
+    idx.search(q[:1], 10, 40)                 # one query: a wide team
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        idx.search(q, 10, 40, out=out)
+    g.replay()
+    torch.cuda.synchronize()
+    got = [o.cpu().numpy() for o in out]
+    got = (got[0].view(np.uint32), got[1], got[2].view(np.uint32), got[3].view(np.uint32), got[4])
+    assert_same(got, oracle.beam_search(X, adj, 3, Q, 10, 40, max_visits=16384))
+    idx.close()

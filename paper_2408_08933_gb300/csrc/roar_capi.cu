@@ -291,7 +291,14 @@ roar_status plan_search(roar_index *idx, int32_t lmax, SearchArgs &a, int &block
         set_error("roar_search: the bipartite-graph search runs one warp per query");
         return ROAR_EINVAL;
     }
-    if (tw == 0) tw = team_for(a, nq, idx->num_sms);
+    if (tw == 0) {
+        tw = team_for(a, nq, idx->num_sms);
+        if (t.hash > 0) {   // a table too large for one-warp teams is refused for any number of queries
+            SearchArgs one = a;
+            one.hash_log2 = t.hash;
+            if (search_blocks_per_sm(one, 1) <= 0) tw = 1;
+        }
+    }
     choose_visited(a, t.hash, tw, lmax, nq, idx->num_sms);
     int bps = search_blocks_per_sm(a, tw);
     if (bps <= 0) {

@@ -151,3 +151,16 @@ def test_a_small_warm_up_is_enough_for_the_staged_gather():
     got = (got[0].view(np.uint32), got[1], got[2].view(np.uint32), got[3].view(np.uint32), got[4])
     assert_same(got, oracle.beam_search(X, adj, 3, Q, 10, 40, max_visits=16384))
     idx.close()
+
+
+@pytest.mark.parametrize("nq", [1, 3000])
+def test_a_table_too_large_for_one_warp_teams_is_refused_for_any_batch(nq):
+    import torch
+
+    rng = np.random.default_rng(10)
+    X, Q, adj = _unit(rng, 1000, 32), _unit(rng, nq, 32), _graph(rng, 1000, 32)
+    idx = dev_index(X, adj, 3)
+    idx.set_hash_log2(15)                     # 4 teams x 128 KB
+    with pytest.raises(Exception, match="shared memory"):
+        idx.search(torch.from_numpy(Q).to("cuda:0"), 10, 40)
+    idx.close()

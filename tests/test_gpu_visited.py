@@ -164,3 +164,24 @@ def test_a_table_too_large_for_one_warp_teams_is_refused_for_any_batch(nq):
     with pytest.raises(Exception, match="shared memory"):
         idx.search(torch.from_numpy(Q).to("cuda:0"), 10, 40)
     idx.close()
+
+
+def test_tuned_wide_teams_allocate_scratch_for_themselves_only():
+    import torch
+
+    n, L = 1_000_000, 40
+    rng = np.random.default_rng(11)
+    X, Q, adj = _unit(rng, n, 8), _unit(rng, 50, 8), _graph(rng, n, 8)
+    idx = dev_index(X, adj, 0)
+    idx.set_tuning(L, 8)
+    q = torch.from_numpy(Q).to("cuda:0")
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    idx.search(q, 10, L)
+    torch.cuda.synchronize()
+    # 32 warps per SM at most, hence 4 teams; a bitmap and a visit log each (allocations come in 2 MB pages, and
+    # torch takes up to 20 MB for the outputs)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    slots = 4 * sms * (n // 8 + 4 * (16384 + 128))
+    assert free - torch.cuda.mem_get_info()[0] <= slots + (64 << 20)
+    idx.close()

@@ -707,7 +707,13 @@ beam_search_kernel(const SearchArgs a) {
     float *sd = reinterpret_cast<float *>(ci + kCandCap);
     uint32_t *si = reinterpret_cast<uint32_t *>(sd + kCandCap);
     uint32_t *htab = si + kCandCap;
-    volatile int *ctl = reinterpret_cast<volatile int *>(htab + H);  // claim, count, size, claim (high half), next node
+    // Control words (claim, count, size, claim's high half, next node): the leader
+    // writes one before a barrier of its team and the others read it after that
+    // barrier. It is written again only past a further barrier, which they reach
+    // when they have read it: count, size and next node past the one after the
+    // scoring or, at a query's end, past the next claim's; the claim past a
+    // round's, or past the one of a skipped query.
+    volatile int *ctl = reinterpret_cast<volatile int *>(htab + H);
     const CompactTable ct(reinterpret_cast<unsigned char *>(htab + H) + kCtlBytes, a);   // used when a.ct_log2 != 0
 
     const int64_t slot = (int64_t)blockIdx.x * TPB + team;
@@ -791,6 +797,7 @@ beam_search_kernel(const SearchArgs a) {
         const int L = serving ? __ldcg(reinterpret_cast<const int *>(rec + d) + 1) : (a.L_arr ? a.L_arr[qi] : a.L);
         const int64_t ooff = serving ? qi * (int64_t)a.ring_kmax : (a.out_off ? a.out_off[qi] : qi * (int64_t)k);
         if (L < 1 || L > lcap || k < 1 || k > L || (serving && k > a.ring_kmax)) {  // bad (k, L): report, skip
+            tsync();   // all have read the claim and the serving record: both may be rewritten now
             if (leader && lane == 0) {
                 if (a.visits) a.visits[qi] = 0;
                 if (a.hops) a.hops[qi] = 0;
@@ -860,7 +867,9 @@ beam_search_kernel(const SearchArgs a) {
 
         for (;;) {
             int cnt = 0;
-            if (leader) {
+            // A team meets only at rounds with rows to score, or at the end: the
+            // leader walks rounds without new rows by itself.
+            while (leader) {
                 uint32_t v = 0;        // the adjacency row to read this round
                 bool have_row = false;
                 int sel2 = -1;         // the second unexpanded entry (same 32-entry block), or -1
@@ -1008,17 +1017,22 @@ beam_search_kernel(const SearchArgs a) {
                     }
                     visits += cnt;
                 }
+                if (TW > 1 && cnt == 0) {
+                    __syncwarp();
+                    continue;
+                }
                 if (lane == 0) {
                     ctl[1] = cnt;
                     ctl[2] = size;
                     if (kHelp) ctl[4] = sel2 >= 0 ? (int)(pi[sel2] & kIdMask) : -1;
                 }
+                break;
             }
             tsync();
             cnt = ctl[1];
             if (cnt < 0) break;
             const int next_v = kHelp ? ctl[4] : -1;
-            if (cnt == 0) continue;
+            if (TW == 1 && cnt == 0) continue;
 
             // Gather + score: warp wt takes row groups wt, wt + TW, ...
             if constexpr (S > 0) {

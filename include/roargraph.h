@@ -201,7 +201,8 @@ roar_status roar_index_set_tombstones(roar_index *idx, const uint32_t *bits);
  *   queries   device [nq][d] FP32.
  *   k, L      1 <= k <= L <= ROAR_MAX_L.
  *   ids       device [nq][k] uint32 out; unfilled slots ROAR_NONE_ID.
- *   dist      device [nq][k] FP32 out (-<q,x>); unfilled slots +inf.
+ *   dist      device [nq][k] FP32 out (-<q,x>); unfilled slots +inf. A sum that
+ *             is NaN (queries or rows that are not finite) counts as +inf.
  *   visits    device [nq] uint32 out (distinct nodes scored), or NULL.
  *   hops      device [nq] uint32 out (expansions), or NULL.
  *   qstatus   device [nq] int32 out: ROAR_OK, ROAR_EOVERFLOW (visit cap hit;

@@ -254,6 +254,10 @@ __device__ __forceinline__ void fma_pair(unsigned long long &s, float q, float x
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(s) : "l"(q2), "l"(x2));
 }
 
+// The distance of a row whose summed product is -v: +inf in place of NaN, so that
+// (distance, id) orders any rows (the ranks of a merge are distinct slots).
+__device__ __forceinline__ float row_distance(float v) { return fminf(v, __int_as_float(0x7f800000)); }
+
 // Distances for rows ids_s[j] (shared, expanded bit ignored), j = first,
 // first + 1, ... in groups of B, groups `step` apart (one warp's share of a
 // team); writes -<q, x> (times the row scale for FP8) to out_s[j].
@@ -334,9 +338,9 @@ __device__ __forceinline__ void score_rows(const void *base, const float *scales
         __syncwarp();
         if (writer && j0 + rr < cnt) {
             if constexpr (DT == 2) {
-                out_s[j0 + rr] = -(sc * mine);
+                out_s[j0 + rr] = row_distance(-(sc * mine));
             } else {
-                out_s[j0 + rr] = -mine;
+                out_s[j0 + rr] = row_distance(-mine);
             }
         }
     }
@@ -421,9 +425,9 @@ __device__ __forceinline__ void score_rows_staged(const void *base, const float 
         if ((lane & (RS - 1)) == 0 && rr < S && j0 + rr < cnt) {
             if constexpr (DT == 2) {
                 const float s8 = scales ? sbuf[(bi & 1) * S + rr] : 1.0f;
-                out_s[j0 + rr] = -(s8 * mine);
+                out_s[j0 + rr] = row_distance(-(s8 * mine));
             } else {
-                out_s[j0 + rr] = -mine;
+                out_s[j0 + rr] = row_distance(-mine);
             }
         }
     }
@@ -625,8 +629,7 @@ __device__ __forceinline__ void take_smallest(const float *pd, uint32_t *pi, int
         for (int i = lane; i < size; i += 32) {
             const uint32_t u = pi[i];
             if (u & kChecked) continue;
-            const float dv = pd[i] + 0.0f;                             // -0 as +0
-            const uint32_t b = dv == dv ? __float_as_uint(dv) : 0x7FC00000u;   // NaN past +inf
+            const uint32_t b = __float_as_uint(pd[i] + 0.0f);          // -0 as +0
             const uint32_t kv = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
             if (kv < key || (kv == key && u < id)) {
                 key = kv;

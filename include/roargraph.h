@@ -90,7 +90,8 @@ const char *roar_last_error(void);
  * Scratch: a 4-byte work counter at creation; on the first search that needs
  * them, per resident warp a visited bitmap of ceil(n/32) words and a log of
  * max_visits + ROAR_MAX_RMAX ids (growing them synchronises the device, so
- * run one search before capturing searches in a CUDA graph).
+ * run one search of that L before capturing searches in a CUDA graph; the
+ * scratch a captured search points at stays until the handle is destroyed).
  * Searches on one handle must not overlap in time (enqueue them on one
  * stream); create one handle per concurrent stream.
  * Errors: ROAR_EINVAL, ROAR_ENOMEM, ROAR_ECUDA.

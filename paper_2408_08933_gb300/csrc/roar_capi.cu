@@ -64,7 +64,8 @@ struct roar_index {
         int bps_cap = 0;
     } tune[6];
     // scratch: one visited bitmap + log per resident warp, replaced by a larger
-    // one on demand; captured plans and servers hold the one they point at
+    // one on demand; plans and servers hold the one they point at, and the
+    // handle holds those that searches in the caller's own graphs point at
     struct Scratch {
         uint32_t *vbits = nullptr;
         uint32_t *vlog = nullptr;
@@ -75,6 +76,7 @@ struct roar_index {
         }
     };
     std::shared_ptr<Scratch> scratch;
+    std::vector<std::shared_ptr<Scratch>> in_graphs;
     int64_t vbits_words = 0;
     int32_t vlog_cap = 0;
     unsigned int *work = nullptr;
@@ -226,8 +228,13 @@ static roar_status ensure_scratch(roar_index *idx, int64_t slots) {
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(e, "ensure_scratch");
     idx->scratch.reset();   // freed here unless a plan or a server still uses it
-    std::shared_ptr<roar_index::Scratch> n(new (std::nothrow) roar_index::Scratch());
-    if (!n) return ROAR_ENOMEM;
+    std::shared_ptr<roar_index::Scratch> n;
+    try {
+        n = std::make_shared<roar_index::Scratch>();
+    } catch (const std::bad_alloc &) {
+        set_error("roar_search: out of host memory");
+        return ROAR_ENOMEM;
+    }
     const size_t bb = (size_t)slots * idx->vbits_words * sizeof(uint32_t);
     e = cudaMalloc(&n->vbits, bb);
     if (e == cudaSuccess) e = cudaMalloc(&n->vlog, (size_t)slots * idx->vlog_cap * sizeof(uint32_t));
@@ -244,6 +251,26 @@ static roar_status ensure_scratch(roar_index *idx, int64_t slots) {
 }
 
 std::shared_ptr<void> hold_scratch(const roar_index *idx) { return idx->scratch; }
+
+// A search on a capturing stream becomes part of a graph the library does not
+// see again: the scratch it points at stays until the handle goes, also when a
+// later search needs a larger one.
+static roar_status hold_for_capture(roar_index *idx, cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {   // (the legacy stream while another one captures)
+        cudaGetLastError();
+        return ROAR_OK;
+    }
+    if (st != cudaStreamCaptureStatusActive) return ROAR_OK;
+    if (!idx->in_graphs.empty() && idx->in_graphs.back() == idx->scratch) return ROAR_OK;
+    try {
+        idx->in_graphs.push_back(idx->scratch);
+    } catch (const std::bad_alloc &) {
+        set_error("roar_search: out of host memory");
+        return ROAR_ENOMEM;
+    }
+    return ROAR_OK;
+}
 
 int tune_bucket(int L) {
     int b = 0;
@@ -351,6 +378,7 @@ extern "C" roar_status roar_search(roar_index *idx, const float *queries, int64_
     SearchArgs a;
     int blocks = 0, tw = 1;
     roar_status st = plan_search(idx, L, a, blocks, tw, nq);
+    if (st == ROAR_OK) st = hold_for_capture(idx, (cudaStream_t)stream);
     if (st != ROAR_OK) return st;
     a.q = queries;
     a.nq = nq;
@@ -474,7 +502,8 @@ extern "C" roar_status roar_search_uneven(roar_index *idx, const float *queries,
     int blocks = 0, tw = 1;
     roar_status st = fill_uneven(idx, queries, nq, k_dev, L_dev, out_off, L_max, order, ids, dist,
                                  visits, hops, qstatus, a, blocks, tw);
-    if (st != ROAR_OK || nq == 0) return st;
+    if (st == ROAR_OK) st = hold_for_capture(idx, (cudaStream_t)stream);
+    if (st != ROAR_OK) return st;
     cudaError_t e = launch_search(a, blocks, tw, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "roar_search_uneven launch");
     return ROAR_OK;

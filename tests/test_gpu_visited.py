@@ -185,3 +185,40 @@ def test_tuned_wide_teams_allocate_scratch_for_themselves_only():
     slots = 4 * sms * (n // 8 + 4 * (16384 + 128))
     assert free - torch.cuda.mem_get_info()[0] <= slots + (64 << 20)
     idx.close()
+
+
+def test_a_captured_search_keeps_its_scratch():
+    # a capture at L = 500, then a search at L = 100 whose launches keep more CTAs resident and replace the scratch
+    import torch
+
+    n, d, r, nq = 20_000, 200, 32, 3000
+    rng = np.random.default_rng(12)
+    X, Q, adj = _unit(rng, n, d), _unit(rng, nq, d), _graph(rng, n, r)
+    idx = dev_index(X, adj, 3)
+    q = torch.from_numpy(Q).to("cuda:0")
+
+    def outputs():
+        return (torch.empty((nq, 10), dtype=torch.int32, device="cuda:0"), torch.empty((nq, 10), device="cuda:0"),
+                *(torch.empty(nq, dtype=torch.int32, device="cuda:0") for _ in range(3)))
+
+    out, other = outputs(), outputs()
+    idx.search(q, 10, 500, out=out)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        idx.search(q, 10, 500, out=out)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    idx.search(q, 10, 100, out=other)
+    torch.cuda.synchronize()
+    # the larger scratch came on top of the graph's: one bitmap and visit log at least for each query of the batch
+    assert free - torch.cuda.mem_get_info()[0] >= nq * (n // 8 + 4 * 16384)
+    for _ in range(2):
+        for o in out:
+            o.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        got = [o.cpu().numpy()[:300] for o in out]
+        got = (got[0].view(np.uint32), got[1], got[2].view(np.uint32), got[3].view(np.uint32), got[4])
+        assert_same(got, oracle.beam_search(X, adj, 3, Q[:300], 10, 500, max_visits=16384))
+    idx.close()

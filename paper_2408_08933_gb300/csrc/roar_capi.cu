@@ -337,18 +337,21 @@ roar_status plan_search(roar_index *idx, int32_t lmax, SearchArgs &a, int &block
     int64_t want = (nq + tpb - 1) / tpb;
     int64_t full = (int64_t)bps * idx->num_sms;
     blocks = (int)std::max<int64_t>(1, std::min(want, full));
-    // Scratch for the widest launch at this L, not only for this one: a warm-up
-    // of a few queries (wide teams, few slots) is enough before a capture of many.
-    // (The staged kernel keeps more CTAs resident than the plain one; a tuned
-    // team stays the same for any number of queries.)
+    // Scratch for the widest launch at this L and tuning, not only for this one:
+    // a warm-up of a few queries (wide teams, few slots) is enough before a
+    // capture of many. (The staged kernel keeps more CTAs resident than the plain
+    // one. A tuned team, table and CTA cap hold for any number of queries, so no
+    // launch needs more slots than they leave.)
     const int team = t.tw ? t.tw : 1;
     SearchArgs one = a;
-    one.hash_log2 = one.ct_log2 = one.staged = 0;
+    one.hash_log2 = std::max(t.hash, 0);
+    one.ct_log2 = one.staged = 0;
     int most = search_blocks_per_sm(one, team);
     if (!bi && search_staged(a.dtype, a.d, team, a.lcap)) {
         one.staged = 1;
         most = std::max(most, search_blocks_per_sm(one, team));
     }
+    if (t.bps_cap > 0) most = std::min(most, t.bps_cap);
     const int64_t widest = (int64_t)most * teams_per_block(team) * idx->num_sms;
     roar_status st = ensure_scratch(idx, std::max(full * tpb, widest));
     if (st != ROAR_OK) return st;

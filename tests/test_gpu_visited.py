@@ -222,3 +222,24 @@ def test_a_captured_search_keeps_its_scratch():
         got = (got[0].view(np.uint32), got[1], got[2].view(np.uint32), got[3].view(np.uint32), got[4])
         assert_same(got, oracle.beam_search(X, adj, 3, Q[:300], 10, 500, max_visits=16384))
     idx.close()
+
+
+@pytest.mark.parametrize("table,cap", [(0, 1), (-1, 2), (13, 0)])
+def test_tuned_caps_and_tables_bound_the_scratch(table, cap):
+    import torch
+
+    n, L = 1_000_000, 40
+    rng = np.random.default_rng(13)
+    X, Q, adj = _unit(rng, n, 8), _unit(rng, 50, 8), _graph(rng, n, 8)
+    idx = dev_index(X, adj, 0)
+    idx.set_tuning(L, 1, table, cap)
+    q = torch.from_numpy(Q).to("cuda:0")
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    idx.search(q, 10, L)
+    torch.cuda.synchronize()
+    # CTAs of 4 teams: as many per SM as the cap says, or as four tables of 32 KB leave in 228 KB: one
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    slots = 4 * max(cap, 1) * sms * (n // 8 + 4 * (16384 + 128))
+    assert free - torch.cuda.mem_get_info()[0] <= slots + (64 << 20)
+    idx.close()

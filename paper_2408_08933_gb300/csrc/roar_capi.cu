@@ -318,42 +318,39 @@ roar_status plan_search(roar_index *idx, int32_t lmax, SearchArgs &a, int &block
         set_error("roar_search: the bipartite-graph search runs one warp per query");
         return ROAR_EINVAL;
     }
-    if (tw == 0) {
-        tw = team_for(a, nq, idx->num_sms);
-        if (t.hash > 0) {   // a table too large for one-warp teams is refused for any number of queries
-            SearchArgs one = a;
-            one.hash_log2 = t.hash;
-            if (search_blocks_per_sm(one, 1) <= 0) tw = 1;
-        }
+    // Scratch for the widest launch at this L and tuning, not only for this one:
+    // a warm-up of a few queries (wide teams, few slots) is enough before a
+    // capture of many. (The staged kernel keeps more CTAs resident than the plain
+    // one. A tuned team, table and CTA cap hold for any number of queries, so no
+    // launch needs more slots than they leave.)
+    const int team = tw ? tw : 1;
+    SearchArgs one = a;
+    one.hash_log2 = std::max(t.hash, 0);
+    int most = search_blocks_per_sm(one, team);
+    if (!bi && search_staged(a.dtype, a.d, team, a.lcap)) {
+        one.staged = 1;
+        most = std::max(most, search_blocks_per_sm(one, team));
+        one.staged = 0;
     }
+    if (t.bps_cap > 0) most = std::min(most, t.bps_cap);
+    const int64_t widest = (int64_t)most * teams_per_block(team) * idx->num_sms;
+    // (A table too large for one-warp teams is refused for any number of queries.)
+    if (tw == 0) tw = widest > 0 ? team_for(one, nq, idx->num_sms) : 1;
     choose_visited(a, t.hash, tw, lmax, nq, idx->num_sms);
     int bps = search_blocks_per_sm(a, tw);
-    if (bps <= 0) {
+    if (bps <= 0 || widest <= 0) {
         set_error("roar_search: this L does not fit in shared memory");
         return ROAR_EINVAL;
     }
     if (t.bps_cap > 0 && bps > t.bps_cap) bps = t.bps_cap;
     const int tpb = teams_per_block(tw);
     int64_t want = (nq + tpb - 1) / tpb;
-    int64_t full = (int64_t)bps * idx->num_sms;
+    // With a table of ids, CTAs of wide teams can hold more teams than those of
+    // one warp (8,192 slots: 6 per SM of two warps, 4 of one): no more run than
+    // there is scratch for.
+    int64_t full = std::max<int64_t>(1, std::min((int64_t)bps * idx->num_sms, widest / tpb));
     blocks = (int)std::max<int64_t>(1, std::min(want, full));
-    // Scratch for the widest launch at this L and tuning, not only for this one:
-    // a warm-up of a few queries (wide teams, few slots) is enough before a
-    // capture of many. (The staged kernel keeps more CTAs resident than the plain
-    // one. A tuned team, table and CTA cap hold for any number of queries, so no
-    // launch needs more slots than they leave.)
-    const int team = t.tw ? t.tw : 1;
-    SearchArgs one = a;
-    one.hash_log2 = std::max(t.hash, 0);
-    one.ct_log2 = one.staged = 0;
-    int most = search_blocks_per_sm(one, team);
-    if (!bi && search_staged(a.dtype, a.d, team, a.lcap)) {
-        one.staged = 1;
-        most = std::max(most, search_blocks_per_sm(one, team));
-    }
-    if (t.bps_cap > 0) most = std::min(most, t.bps_cap);
-    const int64_t widest = (int64_t)most * teams_per_block(team) * idx->num_sms;
-    roar_status st = ensure_scratch(idx, std::max(full * tpb, widest));
+    roar_status st = ensure_scratch(idx, widest);
     if (st != ROAR_OK) return st;
     a.vbits = idx->scratch->vbits;
     a.vbits_words = idx->vbits_words;

@@ -243,3 +243,28 @@ def test_tuned_caps_and_tables_bound_the_scratch(table, cap):
     slots = 4 * max(cap, 1) * sms * (n // 8 + 4 * (16384 + 128))
     assert free - torch.cuda.mem_get_info()[0] <= slots + (64 << 20)
     idx.close()
+
+
+def test_a_small_warm_up_is_enough_with_a_table_of_ids():
+    # 8,192 slots: one CTA of four one-warp teams per SM, but three CTAs of two two-warp teams
+    import torch
+
+    n, d, r, nq = 20_000, 32, 32, 700
+    rng = np.random.default_rng(14)
+    X, Q, adj = _unit(rng, n, d), _unit(rng, nq, d), _graph(rng, n, r)
+    idx = dev_index(X, adj, 3)
+    idx.set_hash_log2(13)
+    q = torch.from_numpy(Q).to("cuda:0")
+    out = (torch.empty((nq, 10), dtype=torch.int32, device="cuda:0"), torch.empty((nq, 10), device="cuda:0"),
+           *(torch.empty(nq, dtype=torch.int32, device="cuda:0") for _ in range(3)))
+    idx.search(q[:1], 10, 40)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        idx.search(q, 10, 40, out=out)
+    g.replay()
+    torch.cuda.synchronize()
+    got = [o.cpu().numpy() for o in out]
+    got = (got[0].view(np.uint32), got[1], got[2].view(np.uint32), got[3].view(np.uint32), got[4])
+    assert_same(got, oracle.beam_search(X, adj, 3, Q, 10, 40, max_visits=16384))
+    idx.close()

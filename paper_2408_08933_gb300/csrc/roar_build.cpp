@@ -42,6 +42,7 @@
 
 namespace roar {
 roar_status cuda_fail(cudaError_t e, const char *what);
+void destroy_index(roar_index *idx);
 void set_error(const char *msg);
 }  // namespace roar
 
@@ -663,7 +664,7 @@ extern "C" roar_status roar_build_index(const float *X_dev, int64_t n, int32_t d
             build_log("enhancement: searched %.0f of %.0f rows (%.1f s)", (double)q0, (double)n,
                       seconds_since(t0));
         }
-        roar_index_destroy(gi);
+        destroy_index(gi);
         cudaFree(pid);
         cudaFree(pdist);
         cudaFree(cand);
@@ -732,7 +733,7 @@ extern "C" roar_status roar_build_index(const float *X_dev, int64_t n, int32_t d
             if (e == cudaSuccess && rc == ROAR_OK)
                 e = cudaMemcpyAsync(r.data(), oi, r.size() * 4, cudaMemcpyDeviceToHost, s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            roar_index_destroy(gi);
+            destroy_index(gi);
             cudaFree(qd);
             cudaFree(oi);
             cudaFree(od);

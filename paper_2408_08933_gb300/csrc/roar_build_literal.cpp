@@ -31,6 +31,7 @@
 
 namespace roar {
 roar_status cuda_fail(cudaError_t e, const char *what);
+void destroy_index(roar_index *idx);
 void set_error(const char *msg);
 }  // namespace roar
 
@@ -234,7 +235,7 @@ extern "C" roar_status roar_build_index_literal(const float *X_dev, int64_t n, i
                 fwd[q0 + i].assign(hk.begin() + (size_t)i * M, hk.begin() + (size_t)i * M + hc[i]);
             }
         }
-        roar_index_destroy(gi);
+        destroy_index(gi);
         cudaFree(pid);
         cudaFree(pd);
         cudaFree(xs);

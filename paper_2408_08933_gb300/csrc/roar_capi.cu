@@ -13,7 +13,7 @@
 #include "roar_internal.cuh"
 
 namespace roar {
-void knn_pool_trim();
+void knn_pool_trim(int dev);
 
 static thread_local char g_last_error[256] = "";
 
@@ -211,13 +211,23 @@ extern "C" roar_status roar_index_set_tombstones(roar_index *idx, const uint32_t
     return ROAR_OK;
 }
 
-extern "C" void roar_index_destroy(roar_index *idx) {
+namespace roar {
+// A handle of the library's own (construction, insertion) goes without emptying
+// the kNN pool, which the calls around it use.
+void destroy_index(roar_index *idx) {
     if (!idx) return;
     cudaDeviceSynchronize();
     cudaFree(idx->work);
     cudaFree(idx->stage);
     delete idx;
-    knn_pool_trim();
+}
+}  // namespace roar
+
+extern "C" void roar_index_destroy(roar_index *idx) {
+    if (!idx) return;
+    const int dev = idx->device;
+    destroy_index(idx);
+    knn_pool_trim(dev);
 }
 
 namespace roar {

@@ -46,6 +46,7 @@
 
 namespace roar {
 roar_status cuda_fail(cudaError_t e, const char *what);
+void destroy_index(roar_index *idx);
 void set_error(const char *msg);
 }  // namespace roar
 
@@ -685,7 +686,7 @@ struct Inserter {
     }
 
     ~Inserter() {
-        if (gi) roar_index_destroy(gi);
+        if (gi) destroy_index(gi);
         cudaFree(dq);
         cudaFree(ddist);
         cudaFree(dids);

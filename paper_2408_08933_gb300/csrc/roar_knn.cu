@@ -301,11 +301,11 @@ static cudaError_t knn_pool(cudaMemPool_t *pool) {
     *pool = g_knn_pools[dev];
     return cudaSuccess;
 }
-// Gives back what the pools hold and no call is using.
-void knn_pool_trim() {
+// Gives back what the device's pool holds and no call is using.
+void knn_pool_trim(int dev) {
+    if (dev < 0 || dev >= kMaxDevices) return;
     std::lock_guard<std::mutex> lock(g_knn_pool_mu);
-    for (cudaMemPool_t p : g_knn_pools)
-        if (p) cudaMemPoolTrimTo(p, 0);
+    if (g_knn_pools[dev]) cudaMemPoolTrimTo(g_knn_pools[dev], 0);
 }
 }  // namespace roar
 

@@ -88,3 +88,22 @@ def test_a_destroyed_index_gives_the_pool_back():
     assert torch.cuda.mem_get_info()[0] - held >= 4 * 3 << 20
     again = _knn(T, X, 50)
     assert np.array_equal(first[0], again[0]) and np.array_equal(first[1], again[1])
+
+
+def test_the_library_s_own_handles_leave_the_pool():
+    import torch
+    from gpu_util import dev_index
+    from test_gpu_insert import CASES, _case
+
+    import paper_2408_08933_gb300 as pkg
+
+    rng = np.random.default_rng(7)
+    X = rng.standard_normal((10_000, 64)).astype(np.float32)
+    _knn(rng.standard_normal((1000, 64)).astype(np.float32), X, 50)
+    B, T, knn, entry, adj, nout, cnt, _ = _case(*CASES[1])
+    Bd, Ad = torch.from_numpy(B).to("cuda:0"), torch.from_numpy(adj.view(np.int32)).to("cuda:0")
+    pkg.insert(Bd, Ad, entry, CASES[1][1], T, knn[:, 0], nout.copy(), cnt.copy(), *CASES[1][2:])   # searches by a handle of its own
+    idx = dev_index(X[:100], np.full((100, 8), 0xFFFFFFFF, np.uint32), 0)
+    held = torch.cuda.mem_get_info()[0]
+    idx.close()
+    assert torch.cuda.mem_get_info()[0] - held >= 4 * 3 << 20     # it was there until the program's handle went

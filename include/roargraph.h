@@ -412,11 +412,19 @@ roar_status roar_quantize(const float *X, int64_t n, int32_t d, roar_dtype dtype
  * rows padded to a multiple of 16 columns, candidate buffers of 3 MB per CTA
  * pair, candidate lists) and synchronises `stream` before returning; scratch of
  * up to 320 MB in all comes from a pool that keeps at most that much per device
- * between calls and gives it back when an index on that device is destroyed.
+ * between calls and gives it back when an index on that device is destroyed,
+ * or by roar_knn_release.
  * Errors: ROAR_EINVAL, ROAR_ENOMEM, ROAR_ECUDA, ROAR_ETIMEOUT (a bounded tensor-core wait gave up).
  */
 roar_status roar_knn(const float *T, int64_t nt, const float *X, int64_t n, int32_t d, int32_t kk,
                      uint32_t *ids, float *dist, void *stream);
+
+/*
+ * Gives back the device memory that roar_knn keeps between calls on the current
+ * device (what a call in another thread is using stays). The next call takes it
+ * again. Errors: ROAR_ECUDA.
+ */
+roar_status roar_knn_release(void);
 
 /*
  * Testing hook of roar_knn's failure handling (no counterpart in the paper):

@@ -98,6 +98,8 @@ def lib() -> ctypes.CDLL:
     L.roar_quantize.restype = ctypes.c_int
     L.roar_knn.argtypes = [P, i64, P, i64, i32, i32, P, P, P]
     L.roar_knn.restype = ctypes.c_int
+    L.roar_knn_release.argtypes = []
+    L.roar_knn_release.restype = ctypes.c_int
     L.roar_knn_set_wait_limit_ns.argtypes = [i64]
     L.roar_knn_set_wait_limit_ns.restype = ctypes.c_int
     L.roar_medoid.argtypes = [P, i64, i32, i32, ctypes.POINTER(u32)]
@@ -270,6 +272,11 @@ def roar_quantize(X, n, d, dtype, out, scales, stream=None):
 
 def roar_knn(T, nt, X, n, d, kk, ids, dist, stream=None):
     _check(lib().roar_knn(T, nt, X, n, d, kk, ids, dist, stream), "roar_knn")
+
+
+def roar_knn_release():
+    """Gives back the device memory that roar_knn keeps between calls on the current device."""
+    _check(lib().roar_knn_release(), "roar_knn_release")
 
 
 def roar_knn_set_wait_limit_ns(ns):

@@ -309,6 +309,14 @@ void knn_pool_trim(int dev) {
 }
 }  // namespace roar
 
+extern "C" roar_status roar_knn_release(void) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_fail(e, "roar_knn_release");
+    knn_pool_trim(dev);
+    return ROAR_OK;
+}
+
 extern "C" roar_status roar_knn(const float *T, int64_t nt, const float *X, int64_t n, int32_t d,
                                 int32_t kk, uint32_t *ids, float *dist, void *stream) {
     constexpr int C = 128;

@@ -107,3 +107,21 @@ def test_the_library_s_own_handles_leave_the_pool():
     held = torch.cuda.mem_get_info()[0]
     idx.close()
     assert torch.cuda.mem_get_info()[0] - held >= 4 * 3 << 20     # it was there until the program's handle went
+
+
+def test_the_pool_is_given_back_on_request():
+    import torch
+
+    import paper_2408_08933_gb300 as pkg
+
+    rng = np.random.default_rng(8)
+    X = rng.standard_normal((10_000, 64)).astype(np.float32)
+    T = rng.standard_normal((1000, 64)).astype(np.float32)
+    first = _knn(T, X, 50)
+    held = torch.cuda.mem_get_info()[0]
+    pkg.roar_knn_release()
+    assert torch.cuda.mem_get_info()[0] - held >= 4 * 3 << 20
+    again = _knn(T, X, 50)
+    assert np.array_equal(first[0], again[0]) and np.array_equal(first[1], again[1])
+    pkg.roar_knn_release()
+    pkg.roar_knn_release()      # nothing left to give

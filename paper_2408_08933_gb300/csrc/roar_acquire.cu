@@ -3,7 +3,7 @@
 // enhancement keep, for node x, the candidates c that are closer to x than to
 // every neighbour already kept).
 //
-// One CTA per node x:
+// One CTA per node x (one warp where there are few candidates):
 //   1. delta(x, c) = -dot(x, c) for every candidate, in the search's fixed FP32
 //      order (score_rows: element i on lane (i >> 2) & 31, fmaf, xor
 //      butterfly), padding ids (0xFFFFFFFF) dropped;
@@ -307,6 +307,135 @@ acquire_kernel(const float *__restrict__ X, int64_t n, int d, const uint32_t *__
     }
 }
 
+// Nodes of few candidates: one warp per node, its own arrays in shared memory,
+// the kept rows read through L1. A CTA per node spends such a node on its
+// barriers. (The rule and its figures: acquire_few_most.)
+constexpr int kAcqFewCand = 40;
+struct AcqFew {                     // per warp
+    float cd[kAcqFewCand], rd[kAcqMaxM];
+    uint32_t ci[kAcqFewCand], res[kAcqMaxM];
+};
+
+__device__ __forceinline__ bool acq_less(float da, uint32_t ia, float db, uint32_t ib) {
+    return da < db || (da == db && ia < ib);
+}
+
+template <int NCH>
+__global__ void __launch_bounds__(128)
+acquire_few_kernel(const float *__restrict__ X, int64_t n, int d, const uint32_t *__restrict__ xs, int64_t nx,
+                   const uint32_t *__restrict__ cand, int cstride, const int32_t *__restrict__ ncand, int M,
+                   int fill, uint32_t *__restrict__ out, int32_t *__restrict__ out_cnt,
+                   uint32_t *__restrict__ sorted_out) {
+    constexpr int B = batch_rows<0, NCH>();
+    __shared__ AcqFew sm[4];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    AcqFew &S = sm[w];
+    const int d4 = d >> 2;
+    for (int64_t i = (int64_t)blockIdx.x * 4 + w; i < nx; i += (int64_t)gridDim.x * 4) {
+        const uint32_t x = xs[i];
+        const int nc = min(max(ncand[i], 0), cstride);
+        const uint32_t *ci_g = cand + (size_t)i * cstride;
+        bool bad = (int64_t)x >= n;
+        int nv = 0;
+        for (int b0 = 0; b0 < nc; b0 += 32) {
+            const int j = b0 + lane;
+            const uint32_t u = j < nc ? ci_g[j] : kNone;
+            const bool ok = u != kNone && (int64_t)u < n;
+            if (u != kNone && !ok) bad = true;
+            const unsigned m = __ballot_sync(kFull, ok);
+            if (ok) S.ci[nv + __popc(m & ((1u << lane) - 1u))] = u;
+            nv += __popc(m);
+        }
+        if (__any_sync(kFull, bad)) {
+            for (int j = lane; j < M; j += 32) out[(size_t)i * M + j] = kNone;
+            if (sorted_out)
+                for (int j = lane; j < cstride; j += 32) sorted_out[(size_t)i * cstride + j] = kNone;
+            if (lane == 0) out_cnt[i] = -1;
+            __syncwarp();
+            continue;
+        }
+        __syncwarp();
+        float4 qr[NCH];
+        load_query<NCH>(X, x, d4, qr, lane);
+        score_rows<0, NCH, B>(X, nullptr, d, d4, qr, S.ci, nv, S.cd, lane);
+        // bitonic sort over the next power of two, padded with (+inf, kNone)
+        int P = 1;
+        while (P < nv) P <<= 1;
+        for (int j = nv + lane; j < P; j += 32) {
+            S.cd[j] = __int_as_float(0x7f800000);
+            S.ci[j] = kNone;
+        }
+        __syncwarp();
+        for (int k = 2; k <= P; k <<= 1) {
+            for (int j = k >> 1; j > 0; j >>= 1) {
+                for (int t = lane; t < P; t += 32) {
+                    const int o = t ^ j;
+                    if (o > t) {
+                        const float da = S.cd[t], db = S.cd[o];
+                        const uint32_t ia = S.ci[t], ib = S.ci[o];
+                        if ((t & k) == 0 ? acq_less(db, ib, da, ia) : acq_less(da, ia, db, ib)) {
+                            S.cd[t] = db;
+                            S.cd[o] = da;
+                            S.ci[t] = ib;
+                            S.ci[o] = ia;
+                        }
+                    }
+                }
+                __syncwarp();
+            }
+        }
+        int nr = 0;
+        auto kept = [&](uint32_t c) {
+            return __any_sync(kFull, (lane < nr && S.res[lane] == c) || (lane + 32 < nr && S.res[lane + 32] == c));
+        };
+        for (int t = 0; t < nv && nr < M; ++t) {
+            const uint32_t c = S.ci[t];
+            if (c == x || kept(c)) continue;
+            if (nr > 0) {
+                float4 qc[NCH];
+                load_query<NCH>(X, c, d4, qc, lane);
+                score_rows<0, NCH, B>(X, nullptr, d, d4, qc, S.res, nr, S.rd, lane);
+                const float dc = S.cd[t];
+                const bool viol = (lane < nr && !(dc < S.rd[lane])) || (lane + 32 < nr && !(dc < S.rd[lane + 32]));
+                if (__any_sync(kFull, viol)) continue;
+            }
+            if (lane == 0) S.res[nr] = c;
+            ++nr;
+            __syncwarp();
+        }
+        if (fill) {
+            for (int t = 0; t < nv && nr < M; ++t) {
+                const uint32_t c = S.ci[t];
+                if (c == x || kept(c)) continue;
+                if (lane == 0) S.res[nr] = c;
+                ++nr;
+                __syncwarp();
+            }
+        }
+        for (int j = lane; j < M; j += 32) out[(size_t)i * M + j] = j < nr ? S.res[j] : kNone;
+        if (sorted_out)
+            for (int j = lane; j < cstride; j += 32) sorted_out[(size_t)i * cstride + j] = j < nv ? S.ci[j] : kNone;
+        if (lane == 0) out_cnt[i] = nr;
+        __syncwarp();
+    }
+}
+
+// The most candidates per node for which one warp per node is the better form (or
+// as good, depending on M and fill). Measured on GB300, one warp per node / one
+// CTA per node, us, M = 16, no fill, 40,000 nodes: d = 200: 8 candidates 98 / 299,
+// 16 449 / 661, 24 744 / 956, 32 1,021 / 1,072, 40 1,374 / 1,260; d = 64: 32 740 / 761,
+// 40 1,020 / 948; d = 512: 24 1,296 / 1,873, 40 2,466 / 2,521, 48 2,993 / 2,642; d =
+// 1024: 8 523 / 854, 16 1,485 / 1,431, 24 2,814 / 2,029 (M = 32 with fill: 16 and
+// 20 candidates 1.16 to 1.3 times as fast for 520 to 1,024 columns). Fewer nodes than
+// warps that run at once are better spread over CTAs: at 100 nodes a CTA is faster
+// from 12 candidates on (d = 200, 24 candidates 36 / 22), at 800 from 32.
+template <int NCH>
+int acquire_few_most(int64_t nx, int sms) {
+    if (nx < 4 * (int64_t)sms) return 8;
+    if (nx < 8 * (int64_t)sms) return NCH >= 8 ? 12 : 24;
+    return NCH >= 8 ? 20 : NCH >= 4 ? kAcqFewCand : 32;
+}
+
 template <int NCH>
 cudaError_t launch_acquire(const float *X, int64_t n, int d, const uint32_t *xs, int64_t nx, const uint32_t *cand,
                            int cstride, const int32_t *ncand, int M, int fill, uint32_t *out, int32_t *out_cnt,
@@ -320,6 +449,12 @@ cudaError_t launch_acquire(const float *X, int64_t n, int d, const uint32_t *xs,
     const size_t smem = (size_t)scap * d * 4 + (size_t)keycap * 8;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess && cstride <= acquire_few_most<NCH>(nx, sms)) {
+        const int64_t few = std::min<int64_t>((nx + 3) / 4, (int64_t)sms * 16);
+        acquire_few_kernel<NCH><<<(unsigned)few, 128, 0, s>>>(X, n, d, xs, nx, cand, cstride, ncand, M, fill, out,
+                                                             out_cnt, sorted_out);
+        return cudaGetLastError();
+    }
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kAcqRowBytes + 8 * kAcqMaxCand);   // any launch's
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, 32 * W, smem);
     if (e != cudaSuccess) return e;

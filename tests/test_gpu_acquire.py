@@ -103,3 +103,31 @@ def test_acquire_close_rows_tie():
     X = np.repeat(X, 8, axis=0)
     X /= np.linalg.norm(X, axis=1, keepdims=True)
     _case(X, 40, [5, 48, 130], 32, True, seed=3)
+
+
+@pytest.mark.parametrize("d", [8, 128, 132, 256, 260, 512, 516, 1024])
+def test_acquire_few_candidates(d):
+    # enough nodes for the warp-per-node form: the oracle's lists, and the same as the CTA-per-node form gives for the
+    # same candidates in wider rows (ties, repeated ids, the node itself, padding and bad ids among them)
+    import torch
+
+    import paper_2408_08933_gb300 as pkg
+
+    rng = np.random.default_rng(d)
+    X = rng.standard_normal((300, d)).astype(np.float32)
+    X /= np.linalg.norm(X, axis=1, keepdims=True)
+    X[100:200] = X[:100]
+    c = 20 if d > 512 else 40 if d > 256 else 32
+    _case(X, 1300, [0, 1, 3, c - 1, c], 17, d % 8 == 4, seed=d)
+    xs = rng.integers(0, 300, 1300).astype(np.int32)
+    cand = rng.integers(0, 300, (1300, c)).astype(np.int32)
+    cand[:, 3], cand[5::50, 2], cand[::7, 1], cand[7::60, 0] = cand[:, 4 % c], xs[5::50], -1, 300
+    count = rng.integers(0, c + 1, 1300).astype(np.int32)
+    wide = np.full((1300, 48), -1, np.int32)
+    wide[:, :c] = cand
+    Xd, xd, nd = (torch.from_numpy(a).to("cuda:0") for a in (X, xs, count))
+    for M, fill in ((1, True), (33, False), (64, True)):
+        few = pkg.acquire(Xd, xd, torch.from_numpy(cand).to("cuda:0"), nd, M, fill, sorted_out=True)
+        cta = pkg.acquire(Xd, xd, torch.from_numpy(wide).to("cuda:0"), nd, M, fill, sorted_out=True)
+        assert torch.equal(few[0], cta[0]) and torch.equal(few[1], cta[1]) and torch.equal(few[2], cta[2][:, :c])
+        assert (few[1] == -1).any() and (few[1] > 0).any()

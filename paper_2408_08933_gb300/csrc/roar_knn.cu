@@ -67,12 +67,31 @@ __global__ void quantize_fp8_kernel(const float *__restrict__ X, int64_t n, int 
         o[i] = (uint8_t)__nv_cvt_float_to_fp8(__fdiv_rn(x[i], s), __NV_SATFINITE, __NV_E4M3);
 }
 
-// The same for 16-byte-aligned rows, bound by HBM: LPR lanes per row (a power of
-// two, so narrow rows fill the warp too), each element read once, 16 bytes per
-// lane and load. Measured on GB300, 1M x 512 to FP8: 486 us (5.3 TB/s) with a
+// The same for 16-byte-aligned rows, bound by HBM: 16 bytes per lane and load, each
+// element read once. Measured on GB300, 1M x 512 to FP8: 486 us (5.3 TB/s) with a
 // second read of the row and one-byte stores, 363 us (7.0 TB/s) so.
 
-// BF16 rows of d4 16-byte chunks into rows of dp4 8-byte ones, zeros past d4.
+__device__ __forceinline__ uint2 to_bf16x4(const float4 &v) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+    return make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
+}
+
+// BF16, m 16-byte chunks: rows need no padding, so they are one array and no lane
+// idles at a row's end. (Lanes dealt to rows, 32 at most, with loads that leave
+// nothing in the caches: 300,000 x 200 67 us, x 256 77, x 512 145, x 1,024 284;
+// an element per lane and load 87, 69, 131, 259; so 53, 67, 130 and 255.)
+__global__ void __launch_bounds__(256) quantize_bf16_flat_kernel(const float4 *__restrict__ X, int64_t m,
+                                                                 uint2 *__restrict__ out) {
+    const int64_t i = (int64_t)blockIdx.x * 512 + threadIdx.x, j = i + 256;
+    float4 v, w;
+    if (i < m) v = __ldg(X + i);
+    if (j < m) w = __ldg(X + j);
+    if (i < m) out[i] = to_bf16x4(v);
+    if (j < m) out[j] = to_bf16x4(w);
+}
+
+// BF16 rows of d4 16-byte chunks into rows of dp4 8-byte ones, zeros past d4: LPR
+// lanes per row (a power of two, so narrow rows fill the warp too).
 template <int LPR>
 __global__ void __launch_bounds__(256) quantize_bf16_vec_kernel(const float4 *__restrict__ X, int64_t n, int d4, int dp4,
                                                                 uint2 *__restrict__ out) {
@@ -83,13 +102,12 @@ __global__ void __launch_bounds__(256) quantize_bf16_vec_kernel(const float4 *__
 #pragma unroll 4
     for (int c = threadIdx.x % LPR; c < dp4; c += LPR) {
         const float4 v = c < d4 ? __ldcs(x + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-        o[c] = make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
+        o[c] = to_bf16x4(v);
     }
 }
 
-// FP8 rows of d4 chunks, at most LPR * NCH, held in registers between the row's
-// maximum and the codes.
+// FP8 rows of d4 chunks on LPR lanes, at most LPR * NCH chunks, held in registers
+// between the row's maximum and the codes.
 template <int LPR, int NCH>
 __global__ void __launch_bounds__(256) quantize_fp8_vec_kernel(const float4 *__restrict__ X, int64_t n, int d4,
                                                                uint32_t *__restrict__ out, float *__restrict__ scales) {
@@ -199,7 +217,8 @@ static cudaError_t quantize_bf16_vec(const float *X, int64_t n, int d, int dp, v
     const int d4 = d / 4, dp4 = dp / 4;
     const float4 *x = reinterpret_cast<const float4 *>(X);
     uint2 *o = reinterpret_cast<uint2 *>(out);
-    if (dp4 <= 8) quantize_bf16_vec_kernel<8><<<(unsigned)((n + 31) / 32), 256, 0, s>>>(x, n, d4, dp4, o);
+    if (dp == d) quantize_bf16_flat_kernel<<<(unsigned)((n * d4 + 511) / 512), 256, 0, s>>>(x, n * d4, o);
+    else if (dp4 <= 8) quantize_bf16_vec_kernel<8><<<(unsigned)((n + 31) / 32), 256, 0, s>>>(x, n, d4, dp4, o);
     else if (dp4 <= 16) quantize_bf16_vec_kernel<16><<<(unsigned)((n + 15) / 16), 256, 0, s>>>(x, n, d4, dp4, o);
     else quantize_bf16_vec_kernel<32><<<(unsigned)((n + 7) / 8), 256, 0, s>>>(x, n, d4, dp4, o);
     return cudaGetLastError();

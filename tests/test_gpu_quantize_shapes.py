@@ -28,3 +28,16 @@ def test_widths_and_alignment(n, d, shift):
     assert np.array_equal(got16.cpu().numpy().view(np.uint16), oracle.quant_bf16(X))
     assert np.array_equal(gs.cpu().numpy(), rs)
     assert np.array_equal(got8.cpu().numpy(), ref8)
+
+
+@pytest.mark.parametrize("n,d", [(1, 4), (127, 4), (128, 4), (129, 4), (511, 4), (512, 4), (513, 4), (1003, 380), (64, 640)])
+def test_bf16_block_edges(n, d):
+    # blocks of 512 chunks of 4 elements: one short, full, one over, many
+    import torch
+
+    import paper_2408_08933_gb300 as pkg
+
+    X = np.random.default_rng(n + d).standard_normal((n, d)).astype(np.float32)
+    got, _ = pkg.quantize(torch.from_numpy(X).to("cuda:0"), "bf16")
+    torch.cuda.synchronize()
+    assert np.array_equal(got.cpu().numpy().view(np.uint16), oracle.quant_bf16(X))

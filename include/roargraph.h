@@ -268,8 +268,9 @@ void roar_plan_destroy(roar_plan *plan);
  * Launch tuning for the beam-width bucket that contains L (L <= 32, 64, 128,
  * 256, 512, 1024): team_warps in {1, 2, 4, 8} warps per query (32..256
  * threads), hash_log2 as in roar_index_set_hash_log2, blocks_per_sm_cap = 0
- * for the occupancy limit. Untuned, a launch takes the widest team with which
- * all its queries are resident at once. Results never depend on the tuning.
+ * for the occupancy limit. Untuned, a launch takes the widest team (two warps at
+ * most for BF16 rows of up to 128 columns) with which all its queries are
+ * resident at once. Results never depend on the tuning.
  * Errors: ROAR_EINVAL.
  */
 roar_status roar_index_set_tuning(roar_index *idx, int32_t L, int32_t team_warps, int32_t hash_log2,

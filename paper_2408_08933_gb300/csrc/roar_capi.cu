@@ -290,13 +290,15 @@ int tune_bucket(int L) {
 
 // Warps per query of an untuned launch: the widest team with which all nq
 // queries are resident at once (more queries run one warp each). Measured on
-// GB300, 1M x 200 FP32, L = 100, teams of 1 / 2 / 4 / 8 warps: 1 query 854 / 711 /
-// 623 / 585 us, 300 queries 1348 / 1073 / 934 / 868, 600 queries 1402 / 1123 /
-// 981 / 1333, 1,200 queries 1447 / 1165 / 1535 / 2259, 2,400 queries 1885 / 2058 /
-// 2669 / 4217.
+// GB300, 1M x 200 FP32, L = 100, teams of 1 / 2 / 4 / 8 warps, us: 1 query 836 / 693 /
+// 599 / 519, 300 queries 1,311 / 1,058 / 908 / 802, 600 queries 1,364 / 1,104 / 954 /
+// 1,246. BF16 rows of up to 128 columns: two warps at most (their kernels keep 80
+// registers, and eight warps a hop's rows in one batch that is mostly empty: 10,000 x
+// 64, L = 100, 1 query 328 / 318 / 365 / 359, 300 queries 423 / 404 / 462 / 458;
+// 100,000 x 100, 300 queries 727 / 645 / 738 / 733).
 static int team_for(const SearchArgs &a, int64_t nq, int sms) {
     if (a.bi_off) return 1;
-    for (int tw = 8; tw > 1; tw /= 2) {
+    for (int tw = a.dtype == 1 && search_nch(a.d) == 1 ? 2 : 8; tw > 1; tw /= 2) {
         if (nq > (int64_t)sms * kMaxWarpsPerSm / tw) continue;
         if (nq <= (int64_t)search_blocks_per_sm(a, tw) * teams_per_block(tw) * sms) return tw;
     }

@@ -827,7 +827,7 @@ knn_tc_kernel(const KnnUnits u, int stages, uint2 *__restrict__ scratch, uint2 *
                 if (!dead) {
                     constexpr int kRows = 2;
 #pragma unroll 1
-                    for (int r = seg * (32 / kSegs); r < (seg + 1) * (32 / kSegs); r += kRows) {
+                    for (int r = seg * (32 / kSegs); r < (seg + 1) * (32 / kSegs) && wrow0 + r < u.nt; r += kRows) {
                         RowList<kSegs> l[kRows];
                         int kept[kRows];
                         float th[kRows];
@@ -848,7 +848,7 @@ knn_tc_kernel(const KnnUnits u, int stages, uint2 *__restrict__ scratch, uint2 *
                 if (__any_sync(kFull, *abort_v != 0)) dead = true;
                 if (!dead) {
                     thr = fmaxf(thr, row_thr[row0 + lane]);
-                    cnt = seg == 0 ? row_kept[row0 + lane] : 0;
+                    cnt = seg == 0 && wrow0 + lane < u.nt ? row_kept[row0 + lane] : 0;   // (no row past the end is trimmed)
                     end = mybuf + 8 * cnt;
                 }
             }

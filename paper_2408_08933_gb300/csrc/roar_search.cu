@@ -75,24 +75,31 @@ void choose_visited(SearchArgs &a, int hash, int tw, int L, int64_t nq, int sms)
         const int64_t need = (nq + (int64_t)tpb * sms - 1) / ((int64_t)tpb * sms);
         const int64_t want = std::min<int64_t>(std::max<int64_t>(need, 1), bps);
         const double est = std::min(visits_for(L), (double)a.n);
-        int lg = 9;
+        // A slot keeps 16 of an id's bits and the bucket stands for the rest, so
+        // sets past 2^21 rows need a table of some size however few the visits
+        // (10M x 64, 10,000 queries, FP32 L = 10 909 us with the bitmap alone, 627
+        // with 4,096 slots; L = 15 1,276 and 860). A full grid of one-warp BF16 / FP8
+        // teams has room for 2,048 slots, hence 8.4M rows; past that the bitmap is
+        // as good as a table of ids for short searches too (FP8 L = 15 1,395 us, a
+        // table of 1,024 ids 1,488).
+        int bits = 1;   // of the ids
+        while (bits < 31 && ((int64_t)1 << bits) < a.n) ++bits;
+        const int least = std::max(9, bits - 16 + kCtBucketLog2);
+        int lg = least;
         while (lg < 15 && (double)(1 << lg) < 2.0 * est) ++lg;
         auto resident = [&](int x) {
             a.ct_log2 = x;
             const size_t smem = search_smem_per_team(a, 0) * tpb;
             return smem > kMaxSmem ? 0 : (int64_t)(228 * 1024 / (smem + 1024));
         };
-        while (lg >= 9 && resident(lg) < want) --lg;
+        while (lg >= least && resident(lg) < want) --lg;
         a.ct_log2 = 0;
-        int bits = 1;   // of the ids
-        while (bits < 31 && ((int64_t)1 << bits) < a.n) ++bits;
         const double bitmaps = (double)std::min<int64_t>(nq, want * tpb * sms) * (double)a.n / 8.0;
         const double share = bitmaps <= 64.0 * (1 << 20) ? 1.5 : 4.0;
-        const int bucket_bits = lg - kCtBucketLog2;
-        if (lg >= 9 && (double)(1 << lg) * share >= est && bits - bucket_bits <= 16) {   // a slot keeps 16 bits
-            if (bits < bucket_bits) bits = bucket_bits;
+        if (lg >= least && lg <= 15 && (double)(1 << lg) * share >= est) {
+            bits = std::max(bits, lg - kCtBucketLog2);
             a.ct_log2 = lg;
-            a.ct_rem = bits - bucket_bits;
+            a.ct_rem = bits - (lg - kCtBucketLog2);
             a.ct_mask = (uint32_t)(((uint64_t)1 << bits) - 1);
         }
     }

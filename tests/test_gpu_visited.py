@@ -268,3 +268,29 @@ def test_a_small_warm_up_is_enough_with_a_table_of_ids():
     got = (got[0].view(np.uint32), got[1], got[2].view(np.uint32), got[3].view(np.uint32), got[4])
     assert_same(got, oracle.beam_search(X, adj, 3, Q, 10, 40, max_visits=16384))
     idx.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "fp8"])
+def test_short_searches_of_sets_past_eight_million_rows(dtype):
+    # 24-bit ids need 2^8 buckets for 16 bits in a slot, more than the visits of these searches ask for
+    n = (1 << 23) + 1000
+    rng = np.random.default_rng(15)
+    X = rng.standard_normal((n, 4), dtype=np.float32)
+    Q = rng.standard_normal((3000, 4), dtype=np.float32)
+    adj = rng.integers(0, n, (n, 8), dtype=np.uint32)
+    adj[:, 7] = adj[:, 0]
+    u = np.arange(n, dtype=np.uint32)
+    special = u[((u * np.uint32(2654435769)) & 0xFFFF) == 0xFFFF]       # the free mark as slot value
+    adj[::3, 5] = rng.choice(special, len(adj[::3]))
+    codes = scales = None
+    if dtype == "bf16":
+        codes = (X.view(np.uint32) >> 16).astype(np.uint16)              # any codes will do
+    elif dtype == "fp8":
+        codes, scales = rng.integers(0, 127, (n, 4), dtype=np.uint8), np.full(n, 0.5, np.float32)
+    kw = {} if dtype == "f32" else {"dtype": dtype, "Xt": codes, "scales": scales}
+    idx = dev_index(X, adj, n - 1, dtype=dtype, trav=codes.view(np.int16) if dtype == "bf16" else codes, scales=scales)
+    for L in (10, 22):
+        ref = oracle.beam_search(X, adj, n - 1, Q, 5, L, max_visits=16384, **kw)
+        for m in (3000, 100):
+            assert_same(run(idx, Q[:m], 5, L), [r[:m] for r in ref], f"L {L}, {m} queries")
+    idx.close()

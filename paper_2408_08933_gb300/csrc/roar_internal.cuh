@@ -129,13 +129,14 @@ __host__ __device__ inline int search_nch(int d) {
     return need <= 1 ? 1 : need <= 2 ? 2 : need <= 4 ? 4 : 8;
 }
 
-// For short searches the one-warp kernels can stage their row gathers in
-// shared memory: two buffers of stage_rows(dtype, NCH) rows per warp (FP32:
-// ROAR_STAGE_ROWS rows for d <= 256, BF16 / FP8: ROAR_STAGE_ROWS_LOWP;
-// proportionally fewer for wider rows). Measured on GB300 (1M x 200), FP32
-// with 4 rows: 3-8 % faster at L = 50-150 and equal at L = 300; for longer
-// pools the extra shared memory costs more occupancy than it gains, so the
-// staged variants run only while lcap <= ROAR_STAGE_MAX_LCAP.
+// For short searches the one-warp FP32 kernels of up to 384 columns can stage
+// their row gathers in shared memory: two buffers of stage_rows(dtype, NCH) rows
+// per warp (ROAR_STAGE_ROWS, half of them past 256 columns; the same for BF16 /
+// FP8 with ROAR_STAGE_ROWS_LOWP). The staged kernels need fewer registers, so
+// five CTAs per SM fit where the others have four. For longer pools the extra
+// shared memory costs more occupancy than it gains (1M x 200: 3-8 % faster at L =
+// 50-150, equal at L = 300, both with the bitmap alone), so they run only while
+// lcap <= ROAR_STAGE_MAX_LCAP. choose_visited says where they are the better ones.
 #ifndef ROAR_STAGE_ROWS
 #define ROAR_STAGE_ROWS 4
 #endif
@@ -155,11 +156,7 @@ __host__ __device__ inline int search_nch(int d) {
 // Bytes of one 4-element row chunk: FP32 16, BF16 8, FP8 4.
 __host__ __device__ constexpr int chunk_bytes(int dtype) { return 16 >> dtype; }
 __host__ __device__ constexpr int stage_rows(int dtype, int nch) {
-    return (dtype == 0 ? ROAR_STAGE_ROWS : ROAR_STAGE_ROWS_LOWP) <= 0 ? 0
-           : nch <= 2 ? (dtype == 0 ? ROAR_STAGE_ROWS : ROAR_STAGE_ROWS_LOWP)
-           : ((dtype == 0 ? ROAR_STAGE_ROWS : ROAR_STAGE_ROWS_LOWP) * 2 / nch > 0
-                  ? (dtype == 0 ? ROAR_STAGE_ROWS : ROAR_STAGE_ROWS_LOWP) * 2 / nch
-                  : 1);
+    return nch > 4 ? 0 : (dtype == 0 ? ROAR_STAGE_ROWS : ROAR_STAGE_ROWS_LOWP) / (nch == 4 ? 2 : 1);
 }
 // Staging bytes per warp for S rows per buffer: two buffers of S rows of d4
 // chunks, then (FP8) two buffers of S row scales; a multiple of 16.
@@ -170,7 +167,7 @@ __host__ __device__ inline size_t stage_bytes(int dtype, int S, int d4) {
 // Rows are copied in 16-byte pieces, so a row's bytes must be a multiple of 16
 // (FP32: any d % 4 == 0; BF16: d % 8 == 0; FP8: d % 16 == 0).
 __host__ __device__ inline bool search_staged(int dtype, int d, int tw, int lcap) {
-    return tw == 1 && search_nch(d) == 2 && lcap <= ROAR_STAGE_MAX_LCAP && stage_rows(dtype, 2) > 0 &&
+    return tw == 1 && d <= 384 && lcap <= ROAR_STAGE_MAX_LCAP && stage_rows(dtype, search_nch(d)) > 0 &&
            ((size_t)d * (4 >> dtype)) % 16 == 0;
 }
 

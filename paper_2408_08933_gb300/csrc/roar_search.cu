@@ -58,10 +58,44 @@ int search_blocks_per_sm(const SearchArgs &a, int tw) {
 // 500 / 1000; fewer on smaller sets).
 static double visits_for(int L) { return 128.0 * std::pow((double)L, 2.0 / 3.0); }
 
+// Whether a launch does better with staged gathers and the bitmap alone than with
+// the compact table (`table`: there is room for one) or with plain gathers. On
+// GB300 one-warp FP32 searches, start with the plain side; us:
+// - queries that fill a fifth CTA per SM but no more, where four leave a second
+//   round: 300,000 x 160, 3,000 queries, L = 100 1,724 / 1,485, L = 320 3,838 / 2,690.
+//   Short searches of narrow rows gain nothing (300,000 x 100, L = 60 equal), nor
+//   does a second round of a few queries unless the searches are long (300,000 x
+//   128, 2,440 queries: L = 100 1,117 / 1,276, L = 320 2,730 / 2,292);
+// - 257 to 384 columns, whose plain batches leave lanes idle: all of one round
+//   (300,000 x 320, L = 100: 1,220 queries 1,679 / 1,588, 3,000 2,571 / 2,029), and
+//   larger launches up to 320 columns while the bitmaps stay in L2 (30,000 x 320,
+//   10,000 queries, L = 200 5,241 / 4,381; 1M x 320 the other way round).
+// Without a table staged gathers pay from 129 columns on, as said at search_staged
+// (d = 100 2.39 / 2.35 ms).
+static bool staged_pays(const SearchArgs &a, int L, int64_t nq, int sms, bool table) {
+    if (a.bi_off || !search_staged(a.dtype, a.d, 1, a.lcap)) return false;
+    SearchArgs plain = a, stg = a;
+    plain.staged = plain.ct_log2 = plain.hash_log2 = 0;
+    stg = plain;
+    stg.staged = 1;
+    const int64_t teams = (int64_t)teams_per_block(1) * sms, four = search_blocks_per_sm(plain, 1) * teams,
+                  five = search_blocks_per_sm(stg, 1) * teams;
+    const int nch = search_nch(a.d);
+    if (!table && nch >= 2) return true;
+    if (nch == 4)
+        return nq <= five || (a.d <= 320 && (double)five * (double)a.n / 8.0 <= 128.0 * (1 << 20));
+    const bool few_more = nq <= four + four / 16 && L <= (nch == 2 ? 128 : 256);
+    return nq > four && nq <= five && !few_more && (nch == 2 || L > 96);
+}
+
 void choose_visited(SearchArgs &a, int hash, int tw, int L, int64_t nq, int sms) {
     a.hash_log2 = hash > 0 ? hash : 0;
     a.ct_log2 = 0;
     a.staged = 0;
+    if (hash == 0 && tw == 1 && staged_pays(a, L, nq, sms, true)) {
+        a.staged = 1;
+        return;
+    }
     if (hash == 0) {
         // The compact table: twice the visits expected, or less, as long as the
         // CTAs this launch can use stay resident. Measured on GB300, 1M rows,
@@ -103,10 +137,9 @@ void choose_visited(SearchArgs &a, int hash, int tw, int L, int64_t nq, int sms)
             a.ct_mask = (uint32_t)(((uint64_t)1 << bits) - 1);
         }
     }
-    // The staged gather pays only without the compact table, whose bytes it
-    // would need (with it 5.1-5.4 ms at L = 100), and for 129 to 256 columns (d =
-    // 512, L = 100: 8.5 ms staged, 7.2 not; d = 100: 2.39, 2.35).
-    if (!a.ct_log2 && !a.bi_off) a.staged = search_staged(a.dtype, a.d, tw, a.lcap) ? 1 : 0;
+    // (With the table the staged gather would need its bytes: 5.1-5.4 ms at 1M x 200,
+    // 10,000 queries, L = 100, 4.99 without it.)
+    if (!a.ct_log2 && tw == 1 && staged_pays(a, L, nq, sms, false)) a.staged = 1;
 }
 
 cudaError_t launch_search(const SearchArgs &a, int blocks, int tw, cudaStream_t s, bool configure) {

@@ -614,6 +614,15 @@ __device__ __forceinline__ int pool_merge(float *pd, uint32_t *pi, int size, int
     return size;
 }
 
+// The same as a call of its own, for the staged kernel of 257 to 384 columns: with
+// the merge inlined the compiler needs half as many instructions again for the
+// rest of a hop there (d = 320, 1,220 queries, L = 100: 2,146 us, 1,665 so).
+__device__ __noinline__ int pool_merge_call(float *pd, uint32_t *pi, int size, int L, const float *cd,
+                                            const uint32_t *ci, int cnt, float *sd, uint32_t *si, int &cursor,
+                                            int lane) {
+    return pool_merge(pd, pi, size, L, cd, ci, cnt, sd, si, cursor, lane);
+}
+
 // Writes the `take` first of a pool's unmarked entries (bit 31 of the id clear;
 // at least that many) in (distance, id) order and marks them. Each lane keeps
 // the first of its own entries (slots lane, lane + 32, ...); per answer the warp
@@ -828,9 +837,10 @@ beam_search_kernel(const SearchArgs a) {
         // second unexpanded entry at selection time is loaded during the hop
         // (a plain load, no side effect); it is the next node expanded unless
         // a new candidate overtakes it, and then its row is already in
-        // registers. (Measured on GB300, 1M x 200: 3 % faster for FP32; the
-        // BF16 / FP8 kernels, short of registers, were slower with it.)
-        constexpr bool kPredict = !BI && DT == 0;
+        // registers. (Measured on GB300, 1M x 200: 3 % faster for FP32; kernels
+        // short of registers are slower with it: BF16 / FP8, and the staged ones:
+        // 300,000 x 200, 3,000 queries, L = 100 1,468 -> 1,432 us without.)
+        constexpr bool kPredict = !BI && DT == 0 && STG == 0;
         constexpr bool kHelp = !BI && TW == 8;
         uint32_t pred_v = kNone;
         uint32_t nbp[kMaxRowPerLane];
@@ -1091,7 +1101,8 @@ beam_search_kernel(const SearchArgs a) {
                 __syncwarp();
                 if (cnt == 0) continue;
             }
-            size = pool_merge(pd, pi, size, L, cd, ci, cnt, sd, si, cursor, lane);
+            if constexpr (STG > 0 && NCH == 4) size = pool_merge_call(pd, pi, size, L, cd, ci, cnt, sd, si, cursor, lane);
+            else size = pool_merge(pd, pi, size, L, cd, ci, cnt, sd, si, cursor, lane);
         }
 
         // Output (re-ranked in FP32, in place, for the reduced-precision forms).
@@ -1190,7 +1201,7 @@ const void *kernel_table(int nch, int rpl, int tw, bool staged) {
 #define ROAR_K(N, R, T) \
     if (nch == N && rpl == R && tw == T && !staged) return (const void *)beam_search_kernel<DT, N, R, T, 0>;
 #define ROAR_KS(N, R)                                                                              \
-    if constexpr (N == 2 && stage_rows(DT, N) > 0) {                                               \
+    if constexpr (stage_rows(DT, N) > 0) {                                                         \
         if (nch == N && rpl == R && tw == 1 && staged)                                             \
             return (const void *)beam_search_kernel<DT, N, R, 1, stage_rows(DT, N)>;               \
     }

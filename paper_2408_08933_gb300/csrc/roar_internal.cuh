@@ -130,20 +130,16 @@ __host__ __device__ inline int search_nch(int d) {
 }
 
 // For short searches the one-warp FP32 kernels of up to 384 columns can stage
-// their row gathers in shared memory: two buffers of stage_rows(dtype, NCH) rows
-// per warp (ROAR_STAGE_ROWS, half of them past 256 columns; the same for BF16 /
-// FP8 with ROAR_STAGE_ROWS_LOWP). The staged kernels need fewer registers, so
-// five CTAs per SM fit where the others have four. For longer pools the extra
-// shared memory costs more occupancy than it gains (1M x 200: 3-8 % faster at L =
-// 50-150, equal at L = 300, both with the bitmap alone), so they run only while
-// lcap <= ROAR_STAGE_MAX_LCAP. choose_visited says where they are the better ones.
+// their row gathers in shared memory: two buffers of stage_rows(NCH) rows per warp
+// (ROAR_STAGE_ROWS, half of them past 256 columns). The staged kernels need fewer
+// registers, so five CTAs per SM fit where the others have four. For longer pools
+// the extra shared memory costs more occupancy than it gains (1M x 200: 3-8 %
+// faster at L = 50-150, equal at L = 300, both with the bitmap alone), so they run
+// only while lcap <= ROAR_STAGE_MAX_LCAP; choose_visited says where they are the
+// better ones. (BF16 / FP8 rows staged so were 5-30 % slower: their plain kernels
+// already gather 8 rows per batch.)
 #ifndef ROAR_STAGE_ROWS
 #define ROAR_STAGE_ROWS 4
-#endif
-// BF16 / FP8 staging is off by default: on GB300 (1M x 200, L = 50-300) it was
-// 5-30 % slower than their register path, which already gathers 8 rows per batch.
-#ifndef ROAR_STAGE_ROWS_LOWP
-#define ROAR_STAGE_ROWS_LOWP 0
 #endif
 #ifndef ROAR_STAGE_MAX_LCAP
 #define ROAR_STAGE_MAX_LCAP 320
@@ -153,22 +149,11 @@ __host__ __device__ inline int search_nch(int d) {
 #ifndef ROAR_MIN_BLOCKS_STAGED
 #define ROAR_MIN_BLOCKS_STAGED 5
 #endif
-// Bytes of one 4-element row chunk: FP32 16, BF16 8, FP8 4.
-__host__ __device__ constexpr int chunk_bytes(int dtype) { return 16 >> dtype; }
-__host__ __device__ constexpr int stage_rows(int dtype, int nch) {
-    return nch > 4 ? 0 : (dtype == 0 ? ROAR_STAGE_ROWS : ROAR_STAGE_ROWS_LOWP) / (nch == 4 ? 2 : 1);
-}
-// Staging bytes per warp for S rows per buffer: two buffers of S rows of d4
-// chunks, then (FP8) two buffers of S row scales; a multiple of 16.
-__host__ __device__ inline size_t stage_bytes(int dtype, int S, int d4) {
-    const size_t b = (size_t)2 * S * d4 * chunk_bytes(dtype) + (dtype == 2 ? (size_t)2 * S * 4 : 0);
-    return (b + 15) / 16 * 16;
-}
-// Rows are copied in 16-byte pieces, so a row's bytes must be a multiple of 16
-// (FP32: any d % 4 == 0; BF16: d % 8 == 0; FP8: d % 16 == 0).
+__host__ __device__ constexpr int stage_rows(int nch) { return nch > 4 ? 0 : ROAR_STAGE_ROWS / (nch == 4 ? 2 : 1); }
+// Staging bytes per warp: two buffers of S rows of d4 16-byte chunks.
+__host__ __device__ inline size_t stage_bytes(int S, int d4) { return (size_t)2 * S * d4 * 16; }
 __host__ __device__ inline bool search_staged(int dtype, int d, int tw, int lcap) {
-    return tw == 1 && d <= 384 && lcap <= ROAR_STAGE_MAX_LCAP && stage_rows(dtype, search_nch(d)) > 0 &&
-           ((size_t)d * (4 >> dtype)) % 16 == 0;
+    return dtype == 0 && tw == 1 && d <= 384 && lcap <= ROAR_STAGE_MAX_LCAP;
 }
 
 constexpr int kCtlBytes = 32;

@@ -31,7 +31,7 @@ static const void *search_kernel(const SearchArgs &a, int tw) {
 }
 
 static size_t stage_of(const SearchArgs &a) {
-    return a.staged ? stage_bytes(a.dtype, stage_rows(a.dtype, search_nch(a.d)), a.d >> 2) : 0;
+    return a.staged ? stage_bytes(stage_rows(search_nch(a.d)), a.d >> 2) : 0;
 }
 
 // Shared memory a CTA can have. A kernel is allowed all of it, never the size

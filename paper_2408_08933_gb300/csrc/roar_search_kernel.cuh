@@ -51,13 +51,6 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
     const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gsrc) : "memory");
 }
-// 4 or 8 bytes global -> shared, asynchronous (cached in L1 and L2).
-template <int N>
-__device__ __forceinline__ void cp_async_small(void *smem_dst, const void *gsrc) {
-    static_assert(N == 4 || N == 8, "cp.async.ca sizes");
-    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(gsrc), "n"(N) : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
@@ -347,29 +340,22 @@ __device__ __forceinline__ void score_rows(const void *base, const float *scales
     __syncwarp();
 }
 
-// Distances for rows ids_s[0..cnt) through shared memory (one warp). The
-// warp copies S rows at a time, in 16-byte pieces (piece p on lane p % 32;
-// for FP8 lane r also the scale of row r), into one of two buffers with
-// cp.async, so the next S rows are in flight while these are scored. After
-// the copies land (each lane waits for its own, then the warp synchronises)
-// every lane reads its chunks (chunk c on lane c % 32, as in score_rows): the
-// decode, the arithmetic and its order are score_rows' exactly. Needs
-// 16-byte-aligned rows (d * element bytes a multiple of 16).
-template <int DT, int NCH, int S>
-__device__ __forceinline__ void score_rows_staged(const void *base, const float *scales, int d4,
-                                                  const float4 (&qr)[NCH], const uint32_t *ids_s, int cnt,
-                                                  float *out_s, int lane, unsigned char *stg) {
-    using Chunk = decltype(RawChunk<DT>::v);
-    constexpr int CB = (int)sizeof(Chunk);
-    static_assert(CB == chunk_bytes(DT), "chunk size");
-    const int rowbytes = d4 * CB;
-    const int pieces = rowbytes >> 4;                 // <= d4 <= 32 * NCH
-    unsigned char *cbuf = stg;
-    float *sbuf = reinterpret_cast<float *>(stg + (size_t)2 * S * rowbytes);   // FP8 row scales
+// Distances for rows ids_s[0..cnt) through shared memory (FP32, one warp). The
+// warp copies S rows at a time, in 16-byte pieces (piece p on lane p % 32), into
+// one of two buffers with cp.async, so the next S rows are in flight while these
+// are scored. After the copies land (each lane waits for its own, then the warp
+// synchronises) every lane reads its chunks (chunk c on lane c % 32, as in
+// score_rows): the arithmetic and its order are score_rows' exactly.
+template <int NCH, int S>
+__device__ __forceinline__ void score_rows_staged(const void *base, int d4, const float4 (&qr)[NCH],
+                                                  const uint32_t *ids_s, int cnt, float *out_s, int lane,
+                                                  unsigned char *stg) {
+    const int rowbytes = d4 * 16;
+    const int pieces = rowbytes >> 4;                 // <= 32 * NCH
     const unsigned char *rows = static_cast<const unsigned char *>(base);
     const int nb = (cnt + S - 1) / S;
     auto issue = [&](int bi) {
-        unsigned char *buf = cbuf + (size_t)(bi & 1) * S * rowbytes;
+        unsigned char *buf = stg + (size_t)(bi & 1) * S * rowbytes;
         const int j0 = bi * S;
 #pragma unroll
         for (int r = 0; r < S; ++r) {
@@ -380,9 +366,6 @@ __device__ __forceinline__ void score_rows_staged(const void *base, const float 
                 for (int c = 0; c < NCH; ++c) {
                     const int p = lane + 32 * c;
                     if (p < pieces) cp_async16(buf + r * rowbytes + p * 16, row + p * 16);
-                }
-                if constexpr (DT == 2) {
-                    if (lane == r && scales) cp_async_small<4>(sbuf + (bi & 1) * S + r, scales + u);
                 }
             }
         }
@@ -398,20 +381,18 @@ __device__ __forceinline__ void score_rows_staged(const void *base, const float 
             cp_async_wait<0>();
         }
         __syncwarp();        // the other lanes' pieces of this batch have landed too
-        const unsigned char *buf = cbuf + (size_t)(bi & 1) * S * rowbytes;
+        const unsigned char *buf = stg + (size_t)(bi & 1) * S * rowbytes;
         const int j0 = bi * S;
         float sc[S];
 #pragma unroll
         for (int r = 0; r < S; ++r) {
             sc[r] = 0.0f;
-            const Chunk *rc = reinterpret_cast<const Chunk *>(buf + r * rowbytes);
+            const float4 *rc = reinterpret_cast<const float4 *>(buf + r * rowbytes);
 #pragma unroll
             for (int c = 0; c < NCH; ++c) {
                 const int ch = lane + 32 * c;
                 if (ch < d4) {
-                    RawChunk<DT> raw;
-                    raw.v = rc[ch];
-                    const float4 x = to_f4<DT>(raw);
+                    const float4 x = rc[ch];
                     sc[r] = fmaf(qr[c].x, x.x, sc[r]);
                     sc[r] = fmaf(qr[c].y, x.y, sc[r]);
                     sc[r] = fmaf(qr[c].z, x.z, sc[r]);
@@ -422,14 +403,7 @@ __device__ __forceinline__ void score_rows_staged(const void *base, const float 
         const float mine = reduce_rows<S>(sc, lane);
         constexpr int RS = reduce_stride<S>();
         const int rr = lane / RS;
-        if ((lane & (RS - 1)) == 0 && rr < S && j0 + rr < cnt) {
-            if constexpr (DT == 2) {
-                const float s8 = scales ? sbuf[(bi & 1) * S + rr] : 1.0f;
-                out_s[j0 + rr] = row_distance(-(s8 * mine));
-            } else {
-                out_s[j0 + rr] = row_distance(-mine);
-            }
-        }
+        if ((lane & (RS - 1)) == 0 && rr < S && j0 + rr < cnt) out_s[j0 + rr] = row_distance(-mine);
     }
     __syncwarp();
 }
@@ -668,7 +642,7 @@ struct TeamShape {
     static constexpr int kThreads = 32 * (TW > kWarpsPerBlock ? TW : kWarpsPerBlock);
     static constexpr int kTeams = kThreads / (32 * TW);
     static constexpr int kWarpBudget =
-        (STG > 0 && DT == 0 ? ROAR_MIN_BLOCKS_STAGED
+        (STG > 0 ? ROAR_MIN_BLOCKS_STAGED
          : TW == 1 && DT == 1 && NCH == 4 ? ROAR_MIN_BLOCKS_BF16_512 : min_blocks_per_sm<DT, NCH>()) *
         kWarpsPerBlock;
     static constexpr int kMinBlocks = (kWarpBudget * 32) / kThreads > 0 ? (kWarpBudget * 32) / kThreads : 1;
@@ -706,9 +680,9 @@ beam_search_kernel(const SearchArgs a) {
     const int lcap = a.lcap;
     const int hlog2 = a.hash_log2;           // 0: no shared table
     const int H = hlog2 ? (1 << hlog2) : 0;
-    static_assert(STG == 0 || TW == 1, "staging is for one-warp kernels");
+    static_assert(STG == 0 || (DT == 0 && TW == 1), "staging is for one-warp FP32 kernels");
     constexpr int S = STG;  // staged gather rows per buffer (0: registers)
-    const size_t stage = S ? stage_bytes(DT, S, a.d >> 2) : 0;
+    const size_t stage = S ? stage_bytes(S, a.d >> 2) : 0;
     unsigned char *tbase = smem_raw + (size_t)team * search_smem_per_team(a, stage);
     unsigned char *stg = tbase + search_smem_per_team(a, 0);
     constexpr int kCandCap = 32 * RPL;
@@ -1049,7 +1023,7 @@ beam_search_kernel(const SearchArgs a) {
 
             // Gather + score: warp wt takes row groups wt, wt + TW, ...
             if constexpr (S > 0) {
-                score_rows_staged<DT, NCH, S>(a.trav, a.scales, d4, qr, ci, cnt, cd, lane, stg);
+                score_rows_staged<NCH, S>(a.trav, d4, qr, ci, cnt, cd, lane, stg);
             } else {
                 score_rows<DT, NCH, B>(a.trav, a.scales, d, d4, qr, ci, cnt, cd, lane, wt * B, TW * B);
             }
@@ -1201,9 +1175,9 @@ const void *kernel_table(int nch, int rpl, int tw, bool staged) {
 #define ROAR_K(N, R, T) \
     if (nch == N && rpl == R && tw == T && !staged) return (const void *)beam_search_kernel<DT, N, R, T, 0>;
 #define ROAR_KS(N, R)                                                                              \
-    if constexpr (stage_rows(DT, N) > 0) {                                                         \
+    if constexpr (DT == 0 && stage_rows(N) > 0) {                                                  \
         if (nch == N && rpl == R && tw == 1 && staged)                                             \
-            return (const void *)beam_search_kernel<DT, N, R, 1, stage_rows(DT, N)>;               \
+            return (const void *)beam_search_kernel<DT, N, R, 1, stage_rows(N)>;                   \
     }
 #define ROAR_KT(N, R) ROAR_K(N, R, 1) ROAR_K(N, R, 2) ROAR_K(N, R, 4) ROAR_K(N, R, 8) ROAR_KS(N, R)
 #define ROAR_KN(N) ROAR_KT(N, 2) ROAR_KT(N, 4)

@@ -311,10 +311,12 @@ acquire_kernel(const float *__restrict__ X, int64_t n, int d, const uint32_t *__
 // the kept rows read through L1. A CTA per node spends such a node on its
 // barriers. (The rule and its figures: acquire_few_most.)
 constexpr int kAcqFewCand = 40;
+constexpr int kAcqFewSlots = 64;    // the sort's: the next power of two
 struct AcqFew {                     // per warp
-    float cd[kAcqFewCand], rd[kAcqMaxM];
-    uint32_t ci[kAcqFewCand], res[kAcqMaxM];
+    float cd[kAcqFewSlots], rd[kAcqMaxM];
+    uint32_t ci[kAcqFewSlots], res[kAcqMaxM];
 };
+static_assert(kAcqFewCand <= kAcqFewSlots, "the padded candidates fit");
 
 __device__ __forceinline__ bool acq_less(float da, uint32_t ia, float db, uint32_t ib) {
     return da < db || (da == db && ia < ib);

@@ -193,8 +193,9 @@ __host__ __device__ constexpr int rerank_rows() {
 template <int DT, int NCH>
 __host__ __device__ constexpr int batch_rows() {
     constexpr int f32 = NCH >= ROAR_BATCH_CHUNKS ? 1 : ROAR_BATCH_CHUNKS / NCH;
-    // BF16 / FP8 rows of 257 to 512 columns (d = 512, L = 350): 4 rows 8.19 / 7.33 ms,
-    // 6 rows 9.13 / 7.94, 8 rows 9.39 / 8.69 (BF16 at its CTAs per SM).
+    // BF16 / FP8 rows of 257 to 512 columns (4,099 queries, d = 512, L = 350, all on
+    // one input; other inputs 8.3-8.6 ms for BF16): 4 rows 8.19 / 7.33 ms, 6 rows
+    // 9.13 / 7.94, 8 rows 9.39 / 8.69 (BF16 at its CTAs per SM).
     if (DT != 0 && NCH == 4) return 4;
     if (DT == 0 && NCH == 2) return 5;   // (L = 90: 4.39 ms; 4, 6, 7, 8 rows 4.52, 4.52, 4.58, 4.65)
     constexpr int lowp = 2 * f32 > ROAR_LOWP_MAX_ROWS ? (f32 > ROAR_LOWP_MAX_ROWS ? f32 : ROAR_LOWP_MAX_ROWS) : 2 * f32;

@@ -430,11 +430,13 @@ acquire_few_kernel(const float *__restrict__ X, int64_t n, int d, const uint32_t
 // 1024: 8 523 / 854, 16 1,485 / 1,431, 24 2,814 / 2,029 (M = 32 with fill: 16 and
 // 20 candidates 1.16 to 1.3 times as fast for 520 to 1,024 columns). Fewer nodes than
 // warps that run at once are better spread over CTAs: at 100 nodes a CTA is faster
-// from 12 candidates on (d = 200, 24 candidates 36 / 22), at 800 from 32.
+// from 12 candidates on (d = 200, 24 candidates 36 / 22), at 800 from 32, at 2,000 from
+// 32 (d = 128, 68 / 53) or 16 (d = 1024, 104 / 85).
 template <int NCH>
 int acquire_few_most(int64_t nx, int sms) {
     if (nx < 4 * (int64_t)sms) return 8;
     if (nx < 8 * (int64_t)sms) return NCH >= 8 ? 12 : 24;
+    if (nx < 16 * (int64_t)sms) return NCH >= 8 ? 12 : NCH >= 2 ? 32 : 24;
     return NCH >= 8 ? 20 : NCH >= 4 ? kAcqFewCand : 32;
 }
 

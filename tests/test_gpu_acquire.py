@@ -118,12 +118,12 @@ def test_acquire_few_candidates(d):
     X /= np.linalg.norm(X, axis=1, keepdims=True)
     X[100:200] = X[:100]
     c = 20 if d > 512 else 40 if d > 256 else 32
-    _case(X, 1300, [0, 1, 3, c - 1, c], 17, d % 8 == 4, seed=d)
-    xs = rng.integers(0, 300, 1300).astype(np.int32)
-    cand = rng.integers(0, 300, (1300, c)).astype(np.int32)
+    _case(X, 2500, [0, 1, 3, c - 1, c], 17, d % 8 == 4, seed=d)
+    xs = rng.integers(0, 300, 2500).astype(np.int32)
+    cand = rng.integers(0, 300, (2500, c)).astype(np.int32)
     cand[:, 3], cand[5::50, 2], cand[::7, 1], cand[7::60, 0] = cand[:, 4 % c], xs[5::50], -1, 300
-    count = rng.integers(0, c + 1, 1300).astype(np.int32)
-    wide = np.full((1300, 48), -1, np.int32)
+    count = rng.integers(0, c + 1, 2500).astype(np.int32)
+    wide = np.full((2500, 48), -1, np.int32)
     wide[:, :c] = cand
     Xd, xd, nd = (torch.from_numpy(a).to("cuda:0") for a in (X, xs, count))
     for M, fill in ((1, True), (33, False), (64, True)):
